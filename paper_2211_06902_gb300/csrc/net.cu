@@ -45,6 +45,13 @@ namespace {
 
 constexpr int NT = 128;
 
+// two neighbouring complex numbers from shared memory (16-byte aligned)
+__device__ __forceinline__ void lds2(const float2* p, float2& a, float2& b) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  a = make_float2(v.x, v.y);
+  b = make_float2(v.z, v.w);
+}
+
 __device__ __forceinline__ int flip_dir(int d) { return d == 0 ? 0 : (d <= 4 ? d + 4 : d - 4); }
 
 // forward layer (also the adjoint, with adjoint weights): output parity p
@@ -368,16 +375,26 @@ __global__ void __launch_bounds__(128, 4) k_ptconv_tc(BatchDev bd, int p, const 
 }
 
 // weight gradient partials: one CTA per (item, rhs) work unit of parity p;
-// partial[unit][d][c][c'] = sum over the unit's sites and colours
+// partial[unit][d][c][c'] = sum over the unit's colours and sites, in that order, in FP32.
+// Per colour a, the 18 warps first lay the transported inputs (T_d phi_c')_a of all nine taps
+// into shared memory (one colour of them is 150 KB at 16 channels), each warp task one tap and
+// 32 sites; then thread (tap, 2 x 2 outputs) runs over the sites with four numbers read per
+// four complex multiply-adds.  Rows are 130 numbers apart: 16-byte reads of eight rows fall
+// into different banks.  Bound by the FP32 pipe and the shared-memory reads of that loop.
+// The form before (one output per thread, rows 128 apart, so the 16 rows of a warp shared
+// one bank, taps one after the other) took 3068 us a layer and parity on 16^4 with 4 rhs, this one
+// 772 us.  Sums run in the order they did, so the gradients are the same to the bit.
+constexpr int WG_THREADS = 576, WG_ROW = NT + 2;
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) k_ptconv_wgrad(BatchDev bd, int p, const float2* __restrict__ in0,
-                                                      const float2* __restrict__ in1,
-                                                      const float2* __restrict__ g0,
-                                                      const float2* __restrict__ g1,
-                                                      float2* __restrict__ partial) {
-  extern __shared__ float2 sm[];
-  float2* sg = sm;                       // [COUT][3][NT]
-  float2* st = sm + COUT * 3 * NT;       // [CIN][3][NT]
+constexpr size_t wgrad_smem() { return sizeof(float2) * (9 * CIN + COUT) * WG_ROW; }
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(WG_THREADS, 1)
+    k_ptconv_wgrad(BatchDev bd, int p, const float2* __restrict__ in0, const float2* __restrict__ in1,
+                   const float2* __restrict__ g0, const float2* __restrict__ g1, float2* __restrict__ partial) {
+  extern __shared__ __align__(16) float2 sm[];
+  float2* st = sm;                          // [9][CIN][WG_ROW]
+  float2* sg = sm + 9 * CIN * WG_ROW;       // [COUT][WG_ROW]
   const int item = blockIdx.x / bd.nrhs, r = blockIdx.x - item * bd.nrhs;
   const int4 it = (p ? bd.items[1] : bd.items[0])[item];
   const int sys = it.x * bd.nrhs + r;
@@ -389,68 +406,101 @@ __global__ void __launch_bounds__(256) k_ptconv_wgrad(BatchDev bd, int p, const 
   const float2* inp = (p ? in1 : in0) + off_p / 4 * CIN;
   const float2* inq = (p ? in0 : in1) + off_q / 4 * CIN;
   const float2* gp = (p ? g1 : g0) + off_p / 4 * COUT;
-  const int s = threadIdx.x;
-  const bool live = s < NT && s < it.z;
-  const int i = it.y + s;
-  if (s < NT)
-    for (int c = 0; c < COUT; ++c)
-      for (int a = 0; a < 3; ++a)
-        sg[(c * 3 + a) * NT + s] = live ? gp[cidx(c * 3 + a, n_out, i)] : make_float2(0.f, 0.f);
   const int* nbr = dp->nbr + (p ? 8LL * n0 : 0);
   const float2* lk = dp->link32;
-  for (int d = 0; d < 9; ++d) {
-    __syncthreads();
-    if (s < NT) {
-      int j = -1;
-      if (live) j = d == 0 ? i : nbr[(d - 1) * n_out + i];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  constexpr int TC = COUT / 2, TP = CIN / 2, TILES = TC * TP;      // 2 x 2 output tiles per tap
+  const bool tile = t < 9 * TILES;
+  const int td = t / TILES, c2 = 2 * ((t % TILES) / TP), p2 = 2 * (t % TP);
+  float2 acc[2][2] = {};
+  for (int a = 0; a < 3; ++a) {
+    for (int task = warp; task < 9 * 4; task += WG_THREADS / 32) {
+      const int d = task >> 2, s = (task & 3) * 32 + lane, i = it.y + s;
+      const bool live = s < it.z;
+      float2* row = st + d * CIN * WG_ROW + s;
+      if (d == 0) {
+        for (int cp = 0; cp < CIN; ++cp)
+          row[cp * WG_ROW] = live ? inp[cidx(cp * 3 + a, n_out, i)] : make_float2(0.f, 0.f);
+        continue;
+      }
+      const int j = live ? nbr[(d - 1) * n_out + i] : -1;
+      const int mu = (d - 1) & 3;
+      const bool fwd = d <= 4;
+      float2 u[3];
+      if (j >= 0)
+        for (int b = 0; b < 3; ++b)
+          u[b] = fwd ? lk[link_block(p, mu, n0, n_out) + cidx(a * 3 + b, n_out, i)]
+                     : lk[link_block(1 - p, mu, n0, n_in) + cidx(b * 3 + a, n_in, j)];
+#pragma unroll 4
       for (int cp = 0; cp < CIN; ++cp) {
-        float2 tv[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        if (j >= 0) {
-          if (d == 0) {
-            for (int a = 0; a < 3; ++a) tv[a] = inp[cidx(cp * 3 + a, n_out, i)];
-          } else {
-            const int mu = (d - 1) & 3;
-            const bool fwd = d <= 4;
-            float2 v[3];
-            for (int a = 0; a < 3; ++a) v[a] = inq[cidx(cp * 3 + a, n_in, j)];
-            for (int a = 0; a < 3; ++a)
-              for (int b2 = 0; b2 < 3; ++b2) {
-                if (fwd) {
-                  float2 u = lk[link_block(p, mu, n0, n_out) + cidx(a * 3 + b2, n_out, i)];
-                  cfma(tv[a], u, v[b2]);
-                } else {
-                  float2 u = lk[link_block(1 - p, mu, n0, n_in) + cidx(b2 * 3 + a, n_in, j)];
-                  cfmac(tv[a], u, v[b2]);
-                }
-              }
+        float2 tv = make_float2(0.f, 0.f);
+        if (j >= 0)
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {
+            const float2 v = inq[cidx(cp * 3 + b, n_in, j)];
+            if (fwd) cfma(tv, u[b], v);
+            else cfmac(tv, u[b], v);
           }
+        row[cp * WG_ROW] = tv;
+      }
+    }
+    for (int e = t; e < COUT * NT; e += WG_THREADS) {
+      const int c = e / NT, s = e % NT;
+      sg[c * WG_ROW + s] = s < it.z ? gp[cidx(c * 3 + a, n_out, it.y + s)] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    if (tile) {
+      const float2* gr = sg + c2 * WG_ROW;
+      const float2* tr = st + (td * CIN + p2) * WG_ROW;
+#pragma unroll 4
+      for (int k = 0; k < NT; k += 2) {
+        float2 gv[2][2], tv[2][2];                                 // [row][site]
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          lds2(gr + h * WG_ROW + k, gv[h][0], gv[h][1]);
+          lds2(tr + h * WG_ROW + k, tv[h][0], tv[h][1]);
         }
-        for (int a = 0; a < 3; ++a) st[(cp * 3 + a) * NT + s] = tv[a];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) cfmac(acc[c][q], tv[q][s], gv[c][s]);   // g * conj(T phi)
       }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < COUT * CIN; t += blockDim.x) {
-      const int c = t / CIN, cp = t % CIN;
-      float2 acc = make_float2(0.f, 0.f);
-      for (int a = 0; a < 3; ++a) {
-        const float2* gr = sg + (c * 3 + a) * NT;
-        const float2* tr = st + (cp * 3 + a) * NT;
-        for (int k = 0; k < NT; ++k) cfmac(acc, tr[k], gr[k]);   // g * conj(T phi)
-      }
-      partial[((long long)blockIdx.x * 9 + d) * COUT * CIN + t] = acc;
-    }
   }
+  if (tile)
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        partial[((long long)blockIdx.x * 9 + td) * COUT * CIN + (c2 + c) * CIN + p2 + q] = acc[c][q];
 }
 
-// sum of the per-unit partials (fixed order, FP64): G[k] for k < n
-__global__ void k_sum_partials(const float2* __restrict__ partial, long long nunit, int n, double2* G) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
+// sum of the per-unit partials (fixed order, FP64): G[k] for k < n.  A CTA sums 32 neighbouring
+// outputs, each warp every 32nd unit (one 256-byte row per load), then the 32 subtotals in order.
+// Bound by HBM (the partials once); one thread per output walking all units took 760 us a layer on
+// average for the 3328 units of 16^4 with 4 rhs, this 123 us.
+__global__ void __launch_bounds__(1024) k_sum_partials(const float2* __restrict__ partial, long long nunit, int n,
+                                                       double2* G) {
+  __shared__ double2 sub[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k = blockIdx.x * 32 + lane;
   double2 a = make_double2(0.0, 0.0);
-  for (long long u = 0; u < nunit; ++u) {
-    float2 v = partial[u * n + k];
-    a.x += v.x;
-    a.y += v.y;
+  if (k < n)
+    for (long long u = warp; u < nunit; u += 32) {
+      const float2 v = partial[u * n + k];
+      a.x += v.x;
+      a.y += v.y;
+    }
+  sub[warp][lane] = a;
+  __syncthreads();
+  if (warp || k >= n) return;
+  a = sub[0][lane];
+  for (int w = 1; w < 32; ++w) {
+    a.x += sub[w][lane].x;
+    a.y += sub[w][lane].y;
   }
   G[k] = a;
 }
@@ -608,17 +658,16 @@ static dd_status launch_wgrad(dd_ctx* c, const Batch& b, const BatchDev& bd, int
                               float2* partial, cudaStream_t s) {
   const unsigned grid = (unsigned)((long long)b.nitems[p] * b.nrhs);
   if (!grid) return DD_OK;
-  const size_t smem = sizeof(float2) * (cin + cout) * 3 * NT;
-  if (cin == 4 && cout == 16) {
-    DD_CUDA(c, cudaFuncSetAttribute(k_ptconv_wgrad<4, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    DD_COUNT_LAUNCH(), k_ptconv_wgrad<4, 16><<<grid, 256, smem, s>>>(bd, p, in0, in1, g0, g1, partial);
-  } else if (cin == 16 && cout == 16) {
-    DD_CUDA(c, cudaFuncSetAttribute(k_ptconv_wgrad<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    DD_COUNT_LAUNCH(), k_ptconv_wgrad<16, 16><<<grid, 256, smem, s>>>(bd, p, in0, in1, g0, g1, partial);
-  } else {
-    DD_CUDA(c, cudaFuncSetAttribute(k_ptconv_wgrad<16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    DD_COUNT_LAUNCH(), k_ptconv_wgrad<16, 4><<<grid, 256, smem, s>>>(bd, p, in0, in1, g0, g1, partial);
-  }
+  auto go = [&](auto kernel, size_t smem) -> dd_status {
+    DD_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DD_COUNT_LAUNCH(), kernel<<<grid, WG_THREADS, smem, s>>>(bd, p, in0, in1, g0, g1, partial);
+    return DD_OK;
+  };
+  dd_status e;
+  if (cin == 4 && cout == 16) e = go(k_ptconv_wgrad<4, 16>, wgrad_smem<4, 16>());
+  else if (cin == 16 && cout == 16) e = go(k_ptconv_wgrad<16, 16>, wgrad_smem<16, 16>());
+  else e = go(k_ptconv_wgrad<16, 4>, wgrad_smem<16, 4>());
+  if (e != DD_OK) return e;
   DD_CUDA(c, cudaGetLastError());
   return DD_OK;
 }
@@ -702,7 +751,7 @@ static dd_status net_loss_grad(dd_ctx* c, dd_net* n, const Batch& b, const Acts&
     if ((e = launch_wgrad(c, b, bd, 1, cin, cout, A.a[l][0], A.a[l][1], Gr.a[l + 1][0], Gr.a[l + 1][1],
                           part + units0 * nw, s)) != DD_OK)
       return e;
-    DD_COUNT_LAUNCH(), k_sum_partials<<<(nw + 127) / 128, 128, 0, s>>>(part, units0 + units1, nw, G + n->woff[l]);
+    DD_COUNT_LAUNCH(), k_sum_partials<<<(nw + 31) / 32, 1024, 0, s>>>(part, units0 + units1, nw, G + n->woff[l]);
     if (l > 0) {
       const float2* Wa = (const float2*)n->d_wadj + n->woff[l];
       for (int p = 0; p < 2; ++p)
