@@ -1378,21 +1378,32 @@ __global__ void k_pack(BatchDev bd, const double2* __restrict__ user, S* __restr
   st_site<12>(dst, fs.np, fs.i, w);
 }
 
+// A site's 12 numbers are 192 contiguous bytes of the caller layout.  Stored by the
+// thread that holds them, every warp store touched 32 half-filled sectors: 820 us for
+// FP32 vectors of 24^4 x 12 rhs (1.84 GB moved).  Here the sites go through shared memory (rows of 13, which
+// spreads the 16-byte stores of 8 lanes over all banks) and leave as 512-byte runs per
+// warp: 345 us for the FP32 vectors. (From double-float vectors the conversion to
+// FP64 is the bound, and the two forms take the same time.)
 template <class S>
-__global__ void k_unpack(BatchDev bd, const S* __restrict__ ve, const S* __restrict__ vo,
-                         double2* __restrict__ user) {
+__global__ void __launch_bounds__(128) k_unpack(BatchDev bd, const S* __restrict__ ve, const S* __restrict__ vo,
+                                                double2* __restrict__ user) {
+  constexpr int ROW = 13;
+  __shared__ double2 buf[128 * ROW];
   const int4 it = bd.fitems[blockIdx.x];
   const int r = blockIdx.y;
-  if (threadIdx.x >= it.z) return;
   const int sys = it.x * bd.nrhs + r;
-  const DomInst* d = bd.inst_tab + bd.inst[it.x];
-  const FieldSite fs = field_site(bd, d, it);
-  double2* dst = user + bd.uoff[sys] + 12LL * fs.f;
-  const S* src = (fs.p ? vo + bd.off[1][sys] : ve + bd.off[0][sys]);
-  typename StoreTraits<S>::C w[12];
-  ld_site<12>(src, fs.np, fs.i, w);
+  if ((int)threadIdx.x < it.z) {
+    const DomInst* d = bd.inst_tab + bd.inst[it.x];
+    const FieldSite fs = field_site(bd, d, it);
+    const S* src = (fs.p ? vo + bd.off[1][sys] : ve + bd.off[0][sys]);
+    typename StoreTraits<S>::C w[12];
+    ld_site<12>(src, fs.np, fs.i, w);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) dst[k] = to_d2(w[k]);
+    for (int k = 0; k < 12; ++k) buf[threadIdx.x * ROW + k] = to_d2(w[k]);
+  }
+  __syncthreads();
+  double2* dst = user + bd.uoff[sys] + 12LL * it.y;
+  for (int e = threadIdx.x; e < 12 * it.z; e += 128) dst[e] = buf[e / 12 * ROW + e % 12];
 }
 
 // start of a solve in one pass: b (caller layout) -> b and r = b at the outer
