@@ -15,6 +15,7 @@
 // A^{-1} of its output site to the hop sum (epilogue in the FP64 stencil), and
 // the right-hand side is multiplied by A^{-1} once.  The even-odd Schur form of
 // that operator is 1 - kappa^2 A_ee^{-1} H_eo A_oo^{-1} H_oe.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <complex>
@@ -276,32 +277,55 @@ __global__ void k_clover_rownorm(const double2* __restrict__ A, const double2* _
   }
 }
 
-// one thread per (site, chirality block): the hermitian-packed FP32 and
-// double-float copies of A^{-1} (diagonal real parts, then the entries above
-// the diagonal row by row)
-__global__ void k_clover_pack(const double2* __restrict__ Ai, float4* __restrict__ t32,
-                              float4* __restrict__ tdf, long long V) {
+// one thread per (site, chirality block): the hermitian-packed double-float copy
+// of A^{-1} (diagonal real parts, then the entries above the diagonal row by row),
+// word q of site g at [q][clov_pos(g)]
+__global__ void k_clover_pack(const double2* __restrict__ Ai, float4* __restrict__ tdf, long long V) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= 2 * V) return;
   const double2* a = Ai + k * 36;
-  float f[36];
-  float4* o = tdf + k * 18;
+  float4* o = tdf + (k & 1) * 18 * V + clov_pos(k >> 1, V);
   for (int q = 0; q < 3; ++q) {
     const float2 d0 = split_d(a[(2 * q) * 7].x), d1 = split_d(a[(2 * q + 1) * 7].x);
-    o[q] = make_float4(d0.x, d0.y, d1.x, d1.y);
+    o[q * V] = make_float4(d0.x, d0.y, d1.x, d1.y);
   }
-  for (int r = 0; r < 6; ++r) f[r] = (float)a[r * 7].x;
-  int z = 6, zq = 3;
+  int zq = 3;
   for (int r = 0; r < 6; ++r)
-    for (int c = r + 1; c < 6; ++c, z += 2, ++zq) {
+    for (int c = r + 1; c < 6; ++c, ++zq) {
       const double2 m = a[r * 6 + c];
-      f[z] = (float)m.x;
-      f[z + 1] = (float)m.y;
       const float2 re = split_d(m.x), im = split_d(m.y);
-      o[zq] = make_float4(re.x, im.x, re.y, im.y);
+      o[zq * V] = make_float4(re.x, im.x, re.y, im.y);
     }
-  float4* o32 = t32 + k * 9;
-  for (int q = 0; q < 9; ++q) o32[q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+}
+
+// the hermitian-packed FP32 copy of A^{-1} on an instance, quarter by quarter of its
+// link bundles: one thread per (quarter, lane, chirality block); lanes past the end
+// of the parity hold zeros
+__global__ void k_clover_bundle(DomInst d, const double2* __restrict__ Ai, float4* __restrict__ out,
+                                long long nquarters) {
+  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nquarters * LB_LANES * 2) return;
+  const int lane = (int)(k % LB_LANES);
+  const int ch = (int)((k / LB_LANES) & 1);
+  const long long qg = k / (2 * LB_LANES);
+  const int n0 = d.n[0];
+  const long long q1 = lb_quarter_base(1, n0);
+  const int p = qg < q1 ? 0 : 1;
+  const long long i = (qg - (p ? q1 : 0)) * LB_LANES + lane;
+  float f[36];
+  for (int e = 0; e < 36; ++e) f[e] = 0.f;
+  if (i < d.n[p]) {
+    const double2* a = Ai + 72LL * d.glob[(p ? n0 : 0) + i] + 36 * ch;
+    for (int r = 0; r < 6; ++r) f[r] = (float)a[r * 7].x;
+    int z = 6;
+    for (int r = 0; r < 6; ++r)
+      for (int c = r + 1; c < 6; ++c, z += 2) {
+        f[z] = (float)a[r * 6 + c].x;
+        f[z + 1] = (float)a[r * 6 + c].y;
+      }
+  }
+  float4* o = out + qg * CLOV_H32_F4 * LB_LANES + ch * 9 * LB_LANES + lane;
+  for (int q = 0; q < 9; ++q) o[q * LB_LANES] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
 }
 
 // v <- A^{-1}(x) v on one parity of a batch of double-float vectors, in FP64
@@ -329,17 +353,33 @@ __global__ void k_clover_apply_df(BatchDev bd, int p, df2s* v, const double2* __
 
 }  // namespace
 
-dd_status clover_mixed_tables(dd_ctx* c) {
+dd_status clover_mixed_tables(dd_ctx* c, const Batch& b) {
   if (!c->clover_ready) return fail(c, DD_EINVAL, "clover term not built");
-  if (c->clover_mixed_ready) return DD_OK;
   dd_status e;
-  if (!c->d_clovi32 && (e = dalloc(c, (void**)&c->d_clovi32, sizeof(float4) * 18ULL * c->V)) != DD_OK) return e;
-  if (!c->d_clovi_df && (e = dalloc(c, (void**)&c->d_clovi_df, sizeof(float4) * 36ULL * c->V)) != DD_OK)
-    return e;
-  DD_COUNT_LAUNCH(), k_clover_pack<<<(unsigned)((2LL * c->V + 127) / 128), 128>>>(c->d_clovi, c->d_clovi32,
-                                                                                  c->d_clovi_df, (long long)c->V);
-  DD_CUDA(c, cudaGetLastError());
-  DD_CUDA(c, cudaDeviceSynchronize());
+  bool built = false;
+  for (int j : b.inst) {
+    Instance& in = c->inst[j];
+    if (in.cb32_buf && in.cb_gen == c->clover_gen) continue;
+    const long long nq = lb_quarter_base(1, in.d.n[0]) + lb_quarter_base(1, in.d.n[1]);
+    if (!in.cb32_buf && (e = dalloc(c, &in.cb32_buf, std::max<size_t>(1, nq) * CLOV_QUARTER_BYTES)) != DD_OK) return e;
+    const long long nt = nq * LB_LANES * 2;
+    if (nt > 0)
+      DD_COUNT_LAUNCH(), k_clover_bundle<<<(unsigned)((nt + 127) / 128), 128>>>(in.d, c->d_clovi, (float4*)in.cb32_buf, nq);
+    DD_CUDA(c, cudaGetLastError());
+    if (in.d.cb32 != (const float4*)in.cb32_buf) c->inst_dirty = true;
+    in.d.cb32 = (const float4*)in.cb32_buf;
+    in.cb_gen = c->clover_gen;
+    built = true;
+  }
+  if (!c->clover_mixed_ready) {
+    if (!c->d_clovi_df && (e = dalloc(c, (void**)&c->d_clovi_df, sizeof(float4) * 36ULL * c->V)) != DD_OK)
+      return e;
+    DD_COUNT_LAUNCH(), k_clover_pack<<<(unsigned)((2LL * c->V + 127) / 128), 128>>>(c->d_clovi, c->d_clovi_df,
+                                                                                    (long long)c->V);
+    DD_CUDA(c, cudaGetLastError());
+    built = true;
+  }
+  if (built) DD_CUDA(c, cudaDeviceSynchronize());
   c->clover_mixed_ready = true;
   return DD_OK;
 }
@@ -360,6 +400,7 @@ dd_status clover_apply_inv_df(dd_ctx* c, const Batch& b, void* ve, void* vo, cud
 dd_status clover_build(dd_ctx* c) {
   c->clover_ready = false;
   c->clover_mixed_ready = false;
+  c->clover_gen += 1;
   if (c->csw == 0.0 || !c->gauge_ready) return DD_OK;
   SigmaBlocks sig;
   if (!sigma_blocks(sig)) return fail(c, DD_EINVAL, "sigma_mu_nu is not chirally block-diagonal");

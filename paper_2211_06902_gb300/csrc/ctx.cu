@@ -163,6 +163,8 @@ void free_instance(Instance& in) {
   dfree(in.linkdf_buf);
   dfree(in.lb32_buf);
   dfree(in.lb16_buf);
+  dfree(in.cb32_buf);
+  in.cb32_buf = nullptr;
   in.glob_buf = in.link64_buf = in.link32_buf = in.link16_buf = in.linkdf_buf = nullptr;
   in.lb32_buf = in.lb16_buf = nullptr;
   in.nbr_buf.reset();
@@ -678,7 +680,6 @@ dd_status dd_destroy(dd_ctx* c) {
   dfree(c->d_err);
   dfree(c->d_clov);
   dfree(c->d_clovi);
-  dfree(c->d_clovi32);
   dfree(c->d_clovi_df);
   free_workspace(c);
   free_plan(c);

@@ -50,6 +50,7 @@ struct DomInst {            // device-visible descriptor (plain data)
   const df2s* linkdf;       // double-float copy (residual of the mixed solver)
   const unsigned char* lb32;  // per-chunk link bundles (FP32 / BF16), see spinor.cuh
   const unsigned char* lb16;
+  const float4* cb32;       // A^{-1} of the clover term per quarter of the link bundles: [quarter][18][lane 32]
 };
 
 // Owning host record of an instance.
@@ -64,6 +65,8 @@ struct Instance {
   void* linkdf_buf = nullptr;
   void* lb32_buf = nullptr;
   void* lb16_buf = nullptr;
+  void* cb32_buf = nullptr;     // clover bundles (clover.cu), of generation cb_gen
+  long long cb_gen = -1;
   std::vector<int> h_glob;      // host copy [p][n_p]
   std::vector<int> h_fmap;      // host copy [p][n_p]
   bool links_ready = false;
@@ -190,11 +193,11 @@ struct dd_ctx {
   double csw = 0.0;
   double2* d_clov = nullptr;
   double2* d_clovi = nullptr;
-  float4* d_clovi32 = nullptr;    // A^{-1} hermitian-packed, FP32 [V][18] float4
-  float4* d_clovi_df = nullptr;   // A^{-1} hermitian-packed, double-float [V][36] float4
+  float4* d_clovi_df = nullptr;   // A^{-1} hermitian-packed, double-float [36][V] float4 (clov_pos order)
+  long long clover_gen = 0;       // counts the builds of A: bundles of another generation are stale
   bool clover_ready = false;
   double clover_cond = 1.0;          // max |A_x|_inf * max |A_x^{-1}|_inf >= cond_2(A)
-  bool clover_mixed_ready = false;   // the two packed tables match A^{-1}
+  bool clover_mixed_ready = false;   // the double-float table matches A^{-1}
   bool clover_active = false;     // inside a solve: every hop applies A^{-1} (clov_inv)
   int* d_err = nullptr;           // [0]: device error word, set by kernels whose bounded waits give up;
                                   // [1]: work-queue counter of the persistent stencil
@@ -262,9 +265,10 @@ struct HopArgs {
   int* err;                 // device error word (bounded waits that gave up)
   const void* clov_inv;     // A^{-1} of the clover term, applied to the hop sum at the output
                             // site (left-preconditioned solves): FP64 [V][72] complex for
-                            // FP64 hops; hermitian-packed FP32 [V][72] floats for FP32 and
-                            // BF16-storage hops; hermitian-packed double-float [V][36]
-                            // float4 for the double-float residual hops
+                            // FP64 hops; hermitian-packed double-float [36][V] float4 for the
+                            // double-float residual hops; for FP32 and BF16-storage hops only
+                            // a flag (their packed FP32 copy is in DomInst::cb32)
+  long long clov_stride;    // V
   int lb_fault;             // test hook of the bundle form (dd_debug_wait_fault): CTA 0 leaves
                             // one quarter's bulk copy unissued and waits a few microseconds
   int* queue;               // work-queue counter of the persistent bundle form
@@ -282,7 +286,9 @@ dd_status gauge_finish(dd_ctx* c);
 dd_status clover_build(dd_ctx* c);
 void gauge_touched(dd_ctx* c);
 dd_status clover_apply(dd_ctx* c, const Batch& b, void* ve, void* vo, bool inverse, cudaStream_t s);
-dd_status clover_mixed_tables(dd_ctx* c);
+// the packed copies of A^{-1} that the mixed solves read: the double-float table and the
+// FP32 bundles of the batch's instances
+dd_status clover_mixed_tables(dd_ctx* c, const Batch& b);
 dd_status clover_apply_inv_df(dd_ctx* c, const Batch& b, void* ve, void* vo, cudaStream_t s);
 
 // layout conversions (stencil.cu)

@@ -928,11 +928,11 @@ dd_status whole_solve(dd_ctx* c, const Batch& b, dd_prec ip, const InnerVecs& w,
   BicgOps<S> ops(c, b, ip, w, st, partial);
   char kb[512];
   snprintf(kb, sizeof kb,
-           "solve:%d:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%a:%a:%a:%a:%d:%d:%d%d%d:%d:%p:%p:%p:%p",
+           "solve:%d:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%p:%a:%a:%a:%a:%d:%d:%d%d%d:%d:%p:%p:%p",
            (int)ip, w.r, w.rhat, w.p, w.v, w.s, w.t, w.x, w.tmp, (void*)st, (void*)partial, (void*)partial_o,
            (void*)d_count, (void*)vrel, rhs, c->kappa, prm->tol, prm->inner_tol, floor_frac, max_outer,
            prm->maxiter, b.hop_variant[0], b.hop_variant[1], b.hop_variant[2], c->clover_active ? 1 : 0,
-           (void*)c->d_clovi32, (void*)c->d_clovi_df, (void*)c->d_inst, vos);
+           (void*)c->d_clovi_df, (void*)c->d_inst, vos);
   const std::string key = std::string(kb) + keyx;
   // kernels per pass of each part (for the launch count), kept with the batch's
   // graphs under the graph's key and a suffix per part
@@ -1084,7 +1084,7 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
     if (prm->flags & (DD_SOLVE_NET_GUESS | DD_SOLVE_NET_PRECOND))
       return fail(c, DD_EINVAL, "the learned network does not include the clover term");
     if (!c->clover_ready && (e = clover_build(c)) != DD_OK) return e;
-    if (ip != DD_F64 && (e = clover_mixed_tables(c)) != DD_OK) return e;
+    if (ip != DD_F64 && (e = clover_mixed_tables(c, b)) != DD_OK) return e;
   }
   // The solve stops on the preconditioned residual A^{-1}(b - D x) relative to
   // A^{-1} b; running it to tol / c_A with c_A >= |A| |A^{-1}| keeps the true

@@ -268,16 +268,18 @@ __device__ __forceinline__ void clover_mul(const double2* __restrict__ M, double
 // hermitian, and so its inverse), so the mixed-precision tables keep half of
 // each 6x6 block.  FP32 packing per chirality block: the 6 real diagonal
 // entries, then the 15 entries above the diagonal (row by row) as complex:
-// 36 floats (144 B), 72 floats per site.
-constexpr int CLOV_H32_FLOATS = 72;
-// (v_ch <- M_ch v_ch for both blocks) from an FP32 packed table
-__device__ __forceinline__ void clover_mul_h(const float4* __restrict__ M, float2 (&v)[12]) {
+// 36 floats (144 B), 18 float4 per site.  The bundle form reads them from shared
+// memory, where a quarter's 18 words of 32 lanes lie lane-fastest.
+constexpr int CLOV_H32_F4 = 18;
+constexpr int CLOV_QUARTER_BYTES = CLOV_H32_F4 * LB_LANES * 16;
+// (v_ch <- M_ch v_ch for both blocks); word q of the site at M[q * LB_LANES]
+__device__ __forceinline__ void clover_mul_h(const float4* M, float2 (&v)[12]) {
 #pragma unroll
   for (int ch = 0; ch < 2; ++ch) {
     float f[36];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-      const float4 t = __ldg(M + ch * 9 + q);
+      const float4 t = M[(ch * 9 + q) * LB_LANES];
       f[4 * q] = t.x;
       f[4 * q + 1] = t.y;
       f[4 * q + 2] = t.z;

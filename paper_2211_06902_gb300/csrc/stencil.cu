@@ -31,15 +31,12 @@ template <>
 __device__ __forceinline__ const df2s* links_of<df2s>(const DomInst& d) { return d.linkdf; }
 
 // A^{-1} of the clover term on the hop sum of output site g: FP64 from the full
-// table, FP32 and double-float from the hermitian-packed tables
-__device__ __forceinline__ void clover_epilogue(const void* t, long long g, double2 (&acc)[12]) {
-  clover_mul((const double2*)t + 72LL * g, acc);
+// table, double-float from the hermitian-packed one
+__device__ __forceinline__ void clover_epilogue(const HopArgs& a, long long g, double2 (&acc)[12]) {
+  clover_mul((const double2*)a.clov_inv + 72LL * g, acc);
 }
-__device__ __forceinline__ void clover_epilogue(const void* t, long long g, float2 (&acc)[12]) {
-  clover_mul_h((const float4*)t + (CLOV_H32_FLOATS / 4) * g, acc);
-}
-__device__ __forceinline__ void clover_epilogue(const void* t, long long g, dfc (&acc)[12]) {
-  clover_mul_h((const float4*)t + CLOV_HDF_F4 * g, acc);
+__device__ __forceinline__ void clover_epilogue(const HopArgs& a, long long g, dfc (&acc)[12]) {
+  clover_mul_h((const float4*)a.clov_inv + clov_pos(g, a.clov_stride), a.clov_stride, acc);
 }
 
 // ROWS: the link is read one row (U) or column (U^+) at a time after the spin
@@ -126,7 +123,7 @@ __device__ __forceinline__ void hop_unit(const BatchDev& bd, const HopArgs& a, l
     // clover term: the hop sum times A^{-1} of the output site (compiled into
     // the FP64 forms and the clover instantiations only)
     if constexpr (CLOV) {
-      if (a.clov_inv) clover_epilogue(a.clov_inv, dp->glob[(p ? n0 : 0) + i], acc);
+      if (a.clov_inv) clover_epilogue(a, dp->glob[(p ? n0 : 0) + i], acc);
     }
     const auto b = mkscal<C>(a.b);
 #pragma unroll
@@ -778,9 +775,10 @@ __device__ __forceinline__ int lb_unit(const BatchDev& bd, const HopArgs& a, int
   typedef typename StoreTraits<S>::C C;
   typedef typename StoreTraits<S>::T T;
   constexpr int QB = lb_quarter_bytes<S>();
+  constexpr int CB = CLOV ? CLOV_QUARTER_BYTES : 0;
   constexpr int NH = LB_QUARTERS / QPC;
   extern __shared__ __align__(128) unsigned char lb_smem[];
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(lb_smem + QPC * QB);
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(lb_smem + QPC * (QB + CB));
   const int p = a.p_out;
   const int item = (int)(unit / (ngroups * NH));
   const int rem = (int)(unit - (long long)item * ngroups * NH);
@@ -821,11 +819,15 @@ __device__ __forceinline__ int lb_unit(const BatchDev& bd, const HopArgs& a, int
       atomicAdd(a.work_bytes, a.site_bytes * min(it.z - q0 * LB_LANES, nq * LB_LANES) * cta_rhs);
     // the bulk copies below overwrite shared memory an earlier unit of this CTA read
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    const unsigned char* src = bundle_of<S>(*dp) +
-        (lb_quarter_base(p, n0) + (long long)LB_QUARTERS * (it.y / LB_CHUNK) + q0) * QB;
+    const long long qg = lb_quarter_base(p, n0) + (long long)LB_QUARTERS * (it.y / LB_CHUNK) + q0;
+    const unsigned char* src = bundle_of<S>(*dp) + qg * QB;
     for (int q = 0; q < nq; ++q) {
-      mbar_expect_tx(&bar[q], QB);
-      if (q != fq) bulk_copy_g2s(lb_smem + q * QB, src + (long long)q * QB, QB, &bar[q]);
+      mbar_expect_tx(&bar[q], QB + CB);
+      if (q != fq) {
+        bulk_copy_g2s(lb_smem + q * QB, src + (long long)q * QB, QB, &bar[q]);
+        if constexpr (CLOV)
+          bulk_copy_g2s(lb_smem + QPC * QB + q * CB, (const unsigned char*)dp->cb32 + (qg + q) * CB, CB, &bar[q]);
+      }
     }
   }
   // Thread 0 waits on every quarter on each path.  If a wait on an issued copy
@@ -868,16 +870,6 @@ __device__ __forceinline__ int lb_unit(const BatchDev& bd, const HopArgs& a, int
     const int li = (q0 + q) * LB_LANES + lane;
     if (li >= it.z) continue;
     const int i = it.y + li;
-    if constexpr (CLOV) {
-      // the site's A^{-1} rows (288 B) into L1 while the eight directions run;
-      // the CTA's other rhs warps then read them from L1 in the epilogue
-      if (w == 0) {
-        const char* t = (const char*)((const float4*)a.clov_inv + (CLOV_H32_FLOATS / 4) * dp->glob[(p ? n0 : 0) + i]);
-#pragma unroll
-        for (int o = 0; o < 288; o += 96) asm volatile("prefetch.global.L1 [%0];" ::"l"(t + o));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(t + 287));
-      }
-    }
     const unsigned char* qb = lb_smem + q * QB;
     const S* ql = reinterpret_cast<const S*>(qb);
     const int* qi = reinterpret_cast<const int*>(qb + lb_link_bytes<S>());
@@ -899,10 +891,10 @@ __device__ __forceinline__ int lb_unit(const BatchDev& bd, const HopArgs& a, int
     hop_lb_dir<4, S, C, RR>(acc, qi, ql, lane, n_in, a.in, off_in, sysk, actk);
     if constexpr (CLOV) {
       // clover term: the hop sums times A^{-1} of the output site
-      const long long gs = dp->glob[(p ? n0 : 0) + i];
+      const float4* M = reinterpret_cast<const float4*>(lb_smem + QPC * QB + q * CLOV_QUARTER_BYTES) + lane;
 #pragma unroll
       for (int k = 0; k < RR; ++k)
-        if (actk[k]) clover_epilogue(a.clov_inv, gs, acc[k]);
+        if (actk[k]) clover_mul_h(M, acc[k]);
     }
 #pragma unroll
     for (int k = 0; k < RR; ++k) {
@@ -1042,7 +1034,8 @@ template <class S, int MINB, int RR, int QPC, int MAXR, bool CLOV = false>
 __global__ void __launch_bounds__(32 * MAXR / RR, MINB)
     k_hop_lb(BatchDev bd, HopArgs a, int ngroups, int rb) {
   extern __shared__ __align__(128) unsigned char lb_smem[];
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(lb_smem + QPC * lb_quarter_bytes<S>());
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(
+      lb_smem + QPC * (lb_quarter_bytes<S>() + (CLOV ? CLOV_QUARTER_BYTES : 0)));
   if (threadIdx.x == 0) {
     for (int q = 0; q < QPC; ++q) mbar_init(&bar[q], 1);
     mbar_fence_init();
@@ -1100,7 +1093,8 @@ static void launch_lb(const BatchDev& bd, const HopArgs& a, long long nitems_p, 
     if (a.dotqs) zero(3);
   }
   DD_COUNT_LAUNCH(), k_hop_lb<S, MINB, RR, QPC, MAXR, CLOV>
-      <<<(unsigned)(nitems_p * ngroups * NH), nthreads, QPC * lb_quarter_bytes<S>() + 64, s>>>(bd, a, ngroups, rb);
+      <<<(unsigned)(nitems_p * ngroups * NH), nthreads,
+         QPC * (lb_quarter_bytes<S>() + (CLOV ? CLOV_QUARTER_BYTES : 0)) + 64, s>>>(bd, a, ngroups, rb);
 }
 
 // the work-queue form: (SMs x MINB) CTAs pull the units from a zeroed counter
@@ -1136,8 +1130,8 @@ void hop_bundle_prepare() {
   const int h32 = 2 * lb_quarter_bytes<float2>() + 64, h16 = 2 * lb_quarter_bytes<__nv_bfloat162>() + 64;
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaFuncSetAttribute(k_hop_lb<float2, 2, 1, 4, 12>, at, b32);
-  cudaFuncSetAttribute(k_hop_lb<float2, 2, 1, 4, 12, true>, at, b32);
-  cudaFuncSetAttribute(k_hop_lb<__nv_bfloat162, 2, 1, 4, 12, true>, at, b16);
+  cudaFuncSetAttribute(k_hop_lb<float2, 2, 1, 2, 12, true>, at, h32 + 2 * CLOV_QUARTER_BYTES);
+  cudaFuncSetAttribute(k_hop_lb<__nv_bfloat162, 2, 1, 2, 12, true>, at, h16 + 2 * CLOV_QUARTER_BYTES);
   cudaFuncSetAttribute(k_hop_lb<float2, 1, 1, 4, 12>, at, b32);
   cudaFuncSetAttribute(k_hop_lb<float2, 2, 2, 4, 12>, at, b32);
   cudaFuncSetAttribute(k_hop_lb<float2, 2, 3, 4, 12>, at, b32);
@@ -1218,9 +1212,10 @@ static void dispatch_hop(dd_prec prec, int v, const BatchDev& bd, const HopArgs&
   }
   if (a.clov_inv) {
     // FP32 / BF16 storage with the clover term: the bundle form with the
-    // epilogue compiled in (no launch-form tuning)
-    if (prec == DD_F32) launch_lb<float2, 2, 1, LB_QUARTERS, LB_MAX_RHS, true>(bd, a, ni, s);
-    else launch_lb<__nv_bfloat162, 2, 1, LB_QUARTERS, LB_MAX_RHS, true>(bd, a, ni, s);
+    // epilogue compiled in (no launch-form tuning).  Half items: the links and
+    // A^{-1} of two quarters (57 KB at FP32) leave room for two CTAs per SM.
+    if (prec == DD_F32) launch_lb<float2, 2, 1, 2, LB_MAX_RHS, true>(bd, a, ni, s);
+    else launch_lb<__nv_bfloat162, 2, 1, 2, LB_MAX_RHS, true>(bd, a, ni, s);
     return;
   }
   const HopVariant& hv = variant_of(prec, v);
@@ -1301,8 +1296,8 @@ dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a0,
   a.err = c->d_err;
   a.clov_inv = nullptr;
   if (c->clover_active)
-    a.clov_inv = prec == DD_F64 ? (const void*)c->d_clovi
-                                : (prec == DD_DF64 ? (const void*)c->d_clovi_df : (const void*)c->d_clovi32);
+    a.clov_inv = prec == DD_DF64 ? (const void*)c->d_clovi_df : (const void*)c->d_clovi;
+  a.clov_stride = c->V;
   a.lb_fault = c->debug_wait_fault ? 1 : 0;
   a.queue = c->d_err + 1;
   int p = a.p_out;
