@@ -274,6 +274,7 @@ struct HopArgs {
   int* queue;               // work-queue counter of the persistent bundle form
 };
 dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a, cudaStream_t s);
+void ensure_nsm(dd_ctx* c);      // c->nsm = SMs of the device
 int hop_variant_count(dd_prec prec);
 // sets the shared-memory attributes of the bundle kernels on the current device
 void hop_bundle_prepare();
@@ -314,6 +315,16 @@ void free_workspace(dd_ctx* c);
 void free_plan(dd_ctx* c);
 dd_status get_batch(dd_ctx* c, dd_domain kind, const int* ids, int nblk, int nrhs, Batch** out);
 dd_status get_batch_insts(dd_ctx* c, const std::vector<int>& inst, int nrhs, Batch** out);
+// The inner BiCGstab of a small batch as one launch of thread-block clusters (cluster.cu):
+// its shape (cs = 0 where the launched form is taken), and the solve (the vectors of krylov.cu's
+// inner solver, at precision prec)
+struct ClusterPlan {
+  int rb, cs;               // right-hand sides and CTAs per cluster
+};
+ClusterPlan cluster_plan(dd_ctx* c, const Batch& b, dd_prec prec);
+dd_status run_cluster(dd_ctx* c, const Batch& b, dd_prec prec, ClusterPlan plan, const void* rhs, void* x, void* r,
+                      void* p, void* v, void* s, void* t, void* tmp, SysState* st, double inner_tol2,
+                      double floor_frac, int maxiter, unsigned seed, cudaStream_t q);
 // Flexible GMRES(m) for the even Schur systems of a batch (fgmres.cu): solves
 // M x_e = rhs_e (x_e at the inner precision, from zero) for the systems still in
 // the outer loop, to max(inner_tol2 |rhs|^2, floor_frac outer2); with `net`, the

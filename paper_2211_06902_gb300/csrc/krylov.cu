@@ -587,6 +587,11 @@ struct BicgOps {
     DD_CUDA(c, cudaGetLastError());
     return DD_OK;
   }
+  // the whole inner solve as one launch (small batches)
+  dd_status cluster(ClusterPlan plan, const void* rhs, double inner_tol2, double floor_frac, int maxiter, cudaStream_t s) {
+    return run_cluster(c, b, prec, plan, rhs, w.x, w.r, w.p, w.v, w.s, w.t, w.tmp, st, inner_tol2, floor_frac, maxiter,
+                       rseed, s);
+  }
   // marks the systems that converged in the last iteration
   void final_check(cudaStream_t s) { DD_COUNT_LAUNCH(), k_sc_check<<<sbl, sth, 0, s>>>(sa, nullptr); }
 };
@@ -597,6 +602,11 @@ dd_status run_bicgstab(dd_ctx* c, const Batch& b, dd_prec prec, const InnerVecs&
                        double inner_tol2, double floor_frac, int maxiter, int check_every,
                        bool use_graph, cudaStream_t s, int* iters_run, bool device_loop = false) {
   BicgOps<S> ops(c, b, prec, w, st, partial);
+  const ClusterPlan plan = cluster_plan(c, b, prec);
+  if (plan.cs) {
+    *iters_run = 0;
+    return ops.cluster(plan, rhs, inner_tol2, floor_frac, maxiter, s);
+  }
   dd_status e0 = ops.init(rhs, inner_tol2, floor_frac, s);
   if (e0 != DD_OK) return e0;
   auto iteration = [&](bool check, cudaStream_t s) -> dd_status { return ops.iteration(d_count, check, s); };
@@ -933,7 +943,8 @@ dd_status whole_solve(dd_ctx* c, const Batch& b, dd_prec ip, const InnerVecs& w,
            (void*)d_count, (void*)vrel, rhs, c->kappa, prm->tol, prm->inner_tol, floor_frac, max_outer,
            prm->maxiter, b.hop_variant[0], b.hop_variant[1], b.hop_variant[2], c->clover_active ? 1 : 0,
            (void*)c->d_clovi_df, (void*)c->d_inst, vos);
-  const std::string key = std::string(kb) + keyx;
+  const ClusterPlan plan = cluster_plan(c, b, ip);     // one-launch inner solves (small batches)
+  const std::string key = std::string(kb) + keyx + ":" + std::to_string(plan.cs);
   // kernels per pass of each part (for the launch count), kept with the batch's
   // graphs under the graph's key and a suffix per part
   struct Counts {
@@ -993,14 +1004,17 @@ dd_status whole_solve(dd_ctx* c, const Batch& b, dd_prec ip, const InnerVecs& w,
     cudaGraph_t body_cycle;
     if ((e = ob.cond(h_cycle, cudaGraphCondTypeIf, 1, &body_cycle)) != DD_OK) return e;
     GraphSeq cb{c, body_cycle, c->capture_stream, {}};
-    cudaGraphConditionalHandle h_inner, h_true;
-    DD_CUDA(c, cudaGraphConditionalHandleCreate(&h_inner, body_cycle, 1, 0));
+    cudaGraphConditionalHandle h_inner{}, h_true;
+    if (!plan.cs) DD_CUDA(c, cudaGraphConditionalHandleCreate(&h_inner, body_cycle, 1, 0));
     DD_CUDA(c, cudaGraphConditionalHandleCreate(&h_true, body_cycle, 1, 0));
     if ((e = cb.capture([&](cudaStream_t q) {
            dd_status r;
-           if ((r = to_inner(q)) != DD_OK || (r = schur_rhs(q)) != DD_OK ||
-               (r = ops.init(rhs, inner_tol2, floor_frac, q)) != DD_OK)
-             return r;
+           if ((r = to_inner(q)) != DD_OK || (r = schur_rhs(q)) != DD_OK) return r;
+           if (plan.cs) {
+             DD_CUDA(c, cudaMemsetAsync(d_iter, 0, sizeof(int), q));
+             return ops.cluster(plan, rhs, inner_tol2, floor_frac, prm->maxiter, q);
+           }
+           if ((r = ops.init(rhs, inner_tol2, floor_frac, q)) != DD_OK) return r;
            DD_CUDA(c, cudaMemsetAsync(d_iter, 0, sizeof(int), q));
            // the inner loop's condition starts at 1 on every pass of the outer loop
            DD_COUNT_LAUNCH(), k_cond_set<<<1, 1, 0, q>>>(nullptr, h_inner);
@@ -1009,20 +1023,22 @@ dd_status whole_solve(dd_ctx* c, const Batch& b, dd_prec ip, const InnerVecs& w,
          })) != DD_OK)
       return e;
     n.pre = cb.kernels;
-    cudaGraph_t body_inner;
-    if ((e = cb.cond(h_inner, cudaGraphCondTypeWhile, 1, &body_inner)) != DD_OK) return e;
-    GraphSeq ib{c, body_inner, c->capture_stream, {}};
-    if ((e = ib.capture([&](cudaStream_t q) {
-           dd_status r = ops.iteration(d_count, true, q);
-           if (r != DD_OK) return r;
-           DD_COUNT_LAUNCH(), k_loop_cond<<<1, 1, 0, q>>>(d_count, d_iter, prm->maxiter, h_inner);
-           DD_CUDA(c, cudaGetLastError());
-           return DD_OK;
-         })) != DD_OK)
-      return e;
-    n.inner = ib.kernels;
+    if (!plan.cs) {
+      cudaGraph_t body_inner;
+      if ((e = cb.cond(h_inner, cudaGraphCondTypeWhile, 1, &body_inner)) != DD_OK) return e;
+      GraphSeq ib{c, body_inner, c->capture_stream, {}};
+      if ((e = ib.capture([&](cudaStream_t q) {
+             dd_status r = ops.iteration(d_count, true, q);
+             if (r != DD_OK) return r;
+             DD_COUNT_LAUNCH(), k_loop_cond<<<1, 1, 0, q>>>(d_count, d_iter, prm->maxiter, h_inner);
+             DD_CUDA(c, cudaGetLastError());
+             return DD_OK;
+           })) != DD_OK)
+        return e;
+      n.inner = ib.kernels;
+    }
     if ((e = cb.capture([&](cudaStream_t q) {
-           ops.final_check(q);
+           if (!plan.cs) ops.final_check(q);
            dd_status r = correct_x(q);
            DD_COUNT_LAUNCH(), k_cond_set<<<1, 1, 0, q>>>(&os->tr, h_true);
            DD_CUDA(c, cudaGetLastError());
@@ -1146,6 +1162,7 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
   dim3 eg(b.nitems[0], b.nrhs), og(b.nitems[1], b.nrhs);
   const double kap = c->kappa;
   const bool has_odd = b.nitems[1] > 0;
+  ensure_nsm(c);
 
   EventPair evs;
   cudaEvent_t ev0 = evs.a, ev1 = evs.b;

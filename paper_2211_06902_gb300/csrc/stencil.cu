@@ -1288,6 +1288,14 @@ static double hop_site_bytes(const Batch& b, size_t cb, int nself) {
   return 12.0 * cb * (2 + nself) + 8.0 * 9.0 * cb / b.nrhs;
 }
 
+void ensure_nsm(dd_ctx* c) {
+  if (c->nsm) return;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (c->nsm <= 0) c->nsm = 1;
+}
+
 dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a0, cudaStream_t s) {
   dd_status st = sync_instances(c);
   if (st != DD_OK) return st;
@@ -1319,12 +1327,7 @@ dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a0,
     a.site_bytes = hop_site_bytes(b, prec_bytes(prec), (a.s1 ? 1 : 0) + (a.s2 ? 1 : 0));
     cudaEventRecord(rec.a, s);
   }
-  if (!c->nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (c->nsm <= 0) c->nsm = 1;
-  }
+  ensure_nsm(c);
   const int pi = (prec == DD_F64 || prec == DD_DF64) ? 0 : (prec == DD_F32 ? 1 : 2);
   const int v = c->forced_variant[pi] >= 0 ? c->forced_variant[pi] : b.hop_variant[pi];
   dispatch_hop(prec, v, bd, a, b.nitems[p], c->nsm, s);
