@@ -69,7 +69,7 @@ struct Instance {
   long long cb_gen = -1;
   std::vector<int> h_glob;      // host copy [p][n_p]
   std::vector<int> h_fmap;      // host copy [p][n_p]
-  bool links_ready = false;
+  unsigned links_fresh = 0;     // bit per precision: that copy holds the current links
 };
 
 struct BlockDesc {
@@ -210,6 +210,7 @@ struct dd_ctx {
   cudaStream_t capture_stream = nullptr;   // private stream for CUDA-graph capture
   int undecomposed = 0;                    // bit m: direction m not decomposed (boxes wrap in m)
   cudaStream_t copy_in = nullptr, copy_out = nullptr;   // host<->device copies of pipelined solves
+  bool links_settled = false;              // no kernel in flight reads copies of an earlier gauge field
   int forced_variant[3] = {-1, -1, -1};    // manual stencil launch variant per precision
   bool debug_wait_fault = false;           // test hook: see dd_debug_wait_fault
 };
