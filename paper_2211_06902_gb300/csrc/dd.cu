@@ -233,29 +233,31 @@ __global__ void k_extract(const int* __restrict__ sys_blk, int blk_fixed, const 
   for (int c = 0; c < 12; ++c) o[c] = make_double2(-s[c].x, -s[c].y);
 }
 
-// S^a (one CTA per block) and partial S^r over the dPi1 sites.
-__global__ void k_action_blocks(const int* __restrict__ grp_begin, const int* __restrict__ dpi_idx,
-                                int n_f, int n_dpi, const double2* __restrict__ u,
-                                const double2* __restrict__ chi, const double2* __restrict__ w,
-                                double* out) {
+// Parts of S^a (the boundary sites of a block) and of S^r (a chunk of the dPi1 sites): CTA
+// (group, field * slices + slice) sums one slice of a group's sites for one field, and the host
+// adds the parts in order.  A CTA per group alone left 16 .. 20 CTAs for an 8^4 or 16^4 lattice
+// (378 us a launch on 16^4 with 4 fields); neighbouring threads now take neighbouring numbers.
+__global__ void __launch_bounds__(256) k_action_blocks(const int* __restrict__ grp_begin, const int* __restrict__ dpi_idx,
+                                                       int slices, int n_dpi, const double2* __restrict__ u,
+                                                       const double2* __restrict__ chi, const double2* __restrict__ w,
+                                                       double* out) {
   __shared__ double red[32];
-  const int a = blockIdx.x;
+  const int a = blockIdx.x, f = blockIdx.y / slices, sl = blockIdx.y % slices;
+  const int k0 = grp_begin[a], n = grp_begin[a + 1] - k0;
+  const int per = (n + slices - 1) / slices;
+  const int e1 = 12 * min(n, (sl + 1) * per);
+  const double2 uk = u[f];
+  const long long fb = (long long)f * n_dpi;
   double acc[1] = {0.0};
-  for (int f = 0; f < n_f; ++f) {
-    const double2 uk = u[f];
-    for (int k = grp_begin[a] + threadIdx.x; k < grp_begin[a + 1]; k += blockDim.x) {
-      const long long base = ((long long)f * n_dpi + dpi_idx[k]) * 12;
-#pragma unroll
-      for (int c = 0; c < 12; ++c) {
-        const double2 x = chi[base + c], y = w[base + c];
-        const double re = uk.x * x.x - uk.y * x.y - y.x;
-        const double im = uk.x * x.y + uk.y * x.x - y.y;
-        acc[0] += re * re + im * im;
-      }
-    }
+  for (int e = 12 * sl * per + threadIdx.x; e < e1; e += 256) {
+    const long long at = (fb + dpi_idx[k0 + e / 12]) * 12 + e % 12;
+    const double2 x = chi[at], y = w[at];
+    const double re = uk.x * x.x - uk.y * x.y - y.x;
+    const double im = uk.x * x.y + uk.y * x.x - y.y;
+    acc[0] += re * re + im * im;
   }
   block_reduce<1>(acc, red);
-  if (threadIdx.x == 0) out[a] = acc[0];
+  if (threadIdx.x == 0) out[(long long)blockIdx.y * gridDim.x + a] = acc[0];
 }
 
 // ---- heat-bath of the multi-boson fields: BLAS-1 on dPi vectors [f][n] ---------
@@ -1217,31 +1219,45 @@ static dd_status mb_action_dev(dd_ctx* c, int n_f, const double* u, const double
   const int nb = (int)c->blocks.size();
   const size_t bytes = 16ULL * n_f * c->info.n_dpi * 12;
   dd_status e;
+  if (!c->geom_ready) return fail(c, DD_EINVAL, "geometry not set");
+  if (!c->gauge_ready) return fail(c, DD_EINVAL, "gauge field not uploaded");
+  WPlan* PP;
+  if ((e = build_plan(c, &PP)) != DD_OK) return e;
+  // slices per (group, field): enough CTAs for the SMs, at least 16 sites each
+  const int ncg = PP->n_cgrp;
+  ensure_nsm(c);
+  auto slices_of = [&](int groups, int sites) {
+    const int want = (4 * c->nsm + groups * n_f - 1) / std::max(1, groups * n_f);
+    return std::max(1, std::min(want, sites / (16 * std::max(1, groups))));
+  };
+  const int slb = slices_of(nb, c->info.n_B), slc = slices_of(ncg, c->info.n_C);
+  const size_t parts_b = (size_t)nb * n_f * slb, parts_c = (size_t)ncg * n_f * slc;
   void *wv, *du, *dS;
   if ((e = workspace(c, 46, bytes, &wv)) || (e = workspace(c, 47, 16ULL * n_f, &du)) ||
-      (e = workspace(c, 48, sizeof(double) * (nb + 1 + 4096), &dS)))
+      (e = workspace(c, 48, sizeof(double) * (parts_b + parts_c), &dS)))
     return e;
   dd_status r = apply_w_dev(c, n_f, din, (double*)wv, prm, s);
   if (r != DD_OK && r != DD_ENOCONV) return r;
   DD_CUDA(c, cudaMemcpyAsync(du, u, 16ULL * n_f, cudaMemcpyHostToDevice, s));
   WPlan& P = *(WPlan*)c->wplan;
-  DD_COUNT_LAUNCH(), k_action_blocks<<<nb, 256, 0, s>>>(P.d_b_grp, P.d_b_dpi, n_f, c->info.n_dpi,
-                                     (const double2*)du, (const double2*)din,
-                                     (const double2*)wv, (double*)dS);
-  if (P.n_cgrp > 0)
-    DD_COUNT_LAUNCH(), k_action_blocks<<<P.n_cgrp, 256, 0, s>>>(P.d_c_grp, P.d_c_dpi, n_f, c->info.n_dpi,
-                                             (const double2*)du, (const double2*)din,
-                                             (const double2*)wv, (double*)dS + nb);
+  DD_COUNT_LAUNCH(), k_action_blocks<<<dim3(nb, n_f * slb), 256, 0, s>>>(
+      P.d_b_grp, P.d_b_dpi, slb, c->info.n_dpi, (const double2*)du, (const double2*)din, (const double2*)wv, (double*)dS);
+  if (ncg > 0)
+    DD_COUNT_LAUNCH(), k_action_blocks<<<dim3(ncg, n_f * slc), 256, 0, s>>>(
+        P.d_c_grp, P.d_c_dpi, slc, c->info.n_dpi, (const double2*)du, (const double2*)din, (const double2*)wv,
+        (double*)dS + parts_b);
   DD_CUDA(c, cudaGetLastError());
-  std::vector<double> h(nb + P.n_cgrp);
+  std::vector<double> h(parts_b + parts_c);
   DD_CUDA(c, cudaMemcpyAsync(h.data(), dS, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, s));
   DD_CUDA(c, cudaStreamSynchronize(s));
   double sb = 0.0, sr = 0.0;
   for (int b = 0; b < nb; ++b) {
-    sb += h[b];
-    if (S_block) S_block[b] = h[b];
+    double sa = 0.0;
+    for (size_t k = b; k < parts_b; k += nb) sa += h[k];
+    sb += sa;
+    if (S_block) S_block[b] = sa;
   }
-  for (int k = 0; k < P.n_cgrp; ++k) sr += h[nb + k];
+  for (size_t k = parts_b; k < h.size(); ++k) sr += h[k];
   *S_r = sr;
   *S = sb + sr;
   return r;
