@@ -27,6 +27,7 @@
 // FP64 reductions follow in fixed order (deterministic).
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -57,119 +58,215 @@ __device__ __forceinline__ int glob_index(const int* x, const int* L) {
   return ((x[0] * L[1] + x[1]) * L[2] + x[2]) * L[3] + x[3];
 }
 
-// Adds the hop from global site y (direction dir seen from x) into acc.
-__device__ void add_exterior_hop(double2 (&acc)[12], int dir, int gx, int gy, const InjectArgs& a,
-                                 int f) {
-  const int mu = dir & 3;
-  const bool fwd = dir < 4;
-  const int q = a.dpi_pos[gy];
-  if (q < 0) return;     // cannot happen for a valid geometry (exterior sites lie on dPi)
-  double2 psi[12];
-  const double2* c = a.chi + ((long long)f * a.n_dpi + q) * 12;
+// A tile of INJ_SITES consecutive sites of a caller-layout source: the hops into them from
+// outside, field by field.  Bound by the FP64 pipe (about 110 FP64 instructions a hop).  Few
+// lanes of a warp have a hop in any one direction, so with one thread per site walking its
+// eight directions each warp ran four or five of them for all its lanes, and looked the
+// neighbours up again for every field.  Here the tile's hops are listed direction by direction
+// once, dense warps take them for each field, forward and backward by the same instructions,
+// into sums in shared memory that leave as whole runs.  24^4 with 12 fields: see the launches.
+constexpr int INJ_SITES = 128;
+constexpr int INJ_ROW = 13;               // 12 numbers of a site, padded
+struct InjectTile {
+  double2 acc[INJ_SITES * INJ_ROW];
+  int code[8 * INJ_SITES];                // site in the tile | backward << 8, direction by direction
+  int q[8 * INJ_SITES];                   // dPi index of the neighbour
+  int lsite[8 * INJ_SITES];               // global site that holds the link
+  unsigned mask[8][INJ_SITES / 32];       // ballots
+};
+
+__device__ __forceinline__ double inj_flip(double v, int sign_bit) {
+  return __hiloint2double(__double2hiint(v) ^ sign_bit, __double2loint(v));
+}
+
+// one listed hop: (1 - gamma_mu) U psi or (1 + gamma_mu) U^+ psi, the second by the first's
+// instructions with the lower spins' signs and the link's imaginary parts flipped
+template <int MU>
+__device__ __forceinline__ void inject_hop(InjectTile& T, int e, const InjectArgs& a, int f) {
+  const int code = T.code[e], site = code & 255;
+  const bool back = code >> 8;
+  const int flip = back ? (int)0x80000000 : 0;
+  const double2* c = a.chi + ((long long)f * a.n_dpi + T.q[e]) * 12;
+  double2 psi[12], h[2][3];
 #pragma unroll
   for (int k = 0; k < 12; ++k) psi[k] = c[k];
-  double2 U[9];
-  const double2* l = a.U + (long long)(fwd ? gx : gy) * 36 + mu * 9;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) U[k] = l[k];
-  switch (dir) {
-    case 0: hop_dir<0, true>(acc, psi, U); break;
-    case 1: hop_dir<1, true>(acc, psi, U); break;
-    case 2: hop_dir<2, true>(acc, psi, U); break;
-    case 3: hop_dir<3, true>(acc, psi, U); break;
-    case 4: hop_dir<0, false>(acc, psi, U); break;
-    case 5: hop_dir<1, false>(acc, psi, U); break;
-    case 6: hop_dir<2, false>(acc, psi, U); break;
-    default: hop_dir<3, false>(acc, psi, U); break;
+  for (int k = 6; k < 12; ++k) psi[k] = make_double2(inj_flip(psi[k].x, flip), inj_flip(psi[k].y, flip));
+  hop_project<MU, true>(psi, h);
+  const double2* l = a.U + (long long)T.lsite[e] * 36 + MU * 9;
+  const int sr = back ? 1 : 3, sc = back ? 3 : 1;
+  double2 u[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) u[k] = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    double2 u0 = make_double2(0.0, 0.0), u1 = u0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      double2 m = l[r * sr + k * sc];
+      m.y = inj_flip(m.y, flip);
+      cfma(u0, m, h[0][k]);
+      cfma(u1, m, h[1][k]);
+    }
+    hop_accum_row<MU, true>(u, r, u0, u1);
   }
+  double2* o = T.acc + site * INJ_ROW;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const double2 v = k < 6 ? u[k] : make_double2(inj_flip(u[k].x, flip), inj_flip(u[k].y, flip));
+    o[k] = cadd(o[k], v);
+  }
+}
+
+// n: sites of the tile; nb(dir, q, lsite): the thread's site has a hop in direction dir; out(f):
+// the tile's first number in field f
+template <class Nb, class Out>
+__device__ __forceinline__ void inject_tile(InjectTile& T, int n, const InjectArgs& a, Nb nb, Out out) {
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  int q[8], ls[8];
+  unsigned has = 0;
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    const bool h = tid < n && nb(d, q[d], ls[d]);
+    has |= (unsigned)h << d;
+    const unsigned m = __ballot_sync(0xffffffffu, h);
+    if (lane == 0) T.mask[d][w] = m;
+  }
+  // a site with both hops of a direction (its neighbours on either side lie outside)
+  const int both = __syncthreads_or((has & (has >> 4) & 15u) != 0);
+  int beg[9];
+  beg[0] = 0;
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    const int d = (o >> 1) + 4 * (o & 1);          // +0, -0, +1, -1, ...
+    int at = beg[o], before = 0;
+#pragma unroll
+    for (int k = 0; k < INJ_SITES / 32; ++k) {
+      const int cnt = __popc(T.mask[d][k]);
+      if (k < w) before += cnt;
+      at += cnt;
+    }
+    beg[o + 1] = at;
+    if (has >> d & 1u) {
+      const int e = beg[o] + before + __popc(T.mask[d][w] & ((1u << lane) - 1u));
+      T.code[e] = tid | (d >> 2) << 8;
+      T.q[e] = q[d];
+      T.lsite[e] = ls[d];
+    }
+  }
+  for (int f = blockIdx.y; f < a.n_f; f += gridDim.y) {
+    for (int e = tid; e < INJ_SITES * INJ_ROW; e += INJ_SITES) T.acc[e] = make_double2(0.0, 0.0);
+    __syncthreads();
+    // direction by direction (the sums into a site stay in that order); forward and backward
+    // together unless a site has both
+    auto run = [&](auto mu, int e0, int e1) {
+      for (int e = e0 + tid; e < e1; e += INJ_SITES) inject_hop<decltype(mu)::value>(T, e, a, f);
+      if (e1 > e0) __syncthreads();
+    };
+    auto dir = [&](auto mu) {
+      constexpr int o = 2 * decltype(mu)::value;
+      if (!both) {
+        run(mu, beg[o], beg[o + 2]);
+      } else {
+        run(mu, beg[o], beg[o + 1]);
+        run(mu, beg[o + 1], beg[o + 2]);
+      }
+    };
+    dir(std::integral_constant<int, 0>{});
+    dir(std::integral_constant<int, 1>{});
+    dir(std::integral_constant<int, 2>{});
+    dir(std::integral_constant<int, 3>{});
+    double2* dst = out(f);
+    for (int e = tid; e < 12 * n; e += INJ_SITES) {
+      const double2 v = T.acc[e / 12 * INJ_ROW + e % 12];
+      dst[e] = make_double2(-a.kappa * v.x, -a.kappa * v.y);
+    }
+    __syncthreads();
+  }
+}
+// grid of an injection: tiles x (fields of a batch: as many CTAs as fill the SMs, the rest
+// of the fields one after the other, so the neighbours are looked up once) x instances
+static dim3 inject_grid(dd_ctx* c, int max_sites, int n_f, int nb) {
+  ensure_nsm(c);
+  const int tiles = (max_sites + INJ_SITES - 1) / INJ_SITES;
+  const long long fill = (16LL * c->nsm + (long long)tiles * nb - 1) / std::max(1LL, (long long)tiles * nb);
+  return dim3(tiles, (unsigned)std::max(1LL, std::min<long long>(n_f, fill)), nb);
 }
 
 // Sources for the Omega blocks: s(x) = D_{Omega, ext} chi, x in the box.
-// grid: (ceil(max_sites/128), n_f, nblk)
-__global__ void k_inject_omega(BatchDev bd, InjectArgs a) {
-  const int f = blockIdx.y, j = blockIdx.z;
-  const int sys = j * a.n_f + f;
+__global__ void __launch_bounds__(INJ_SITES) k_inject_omega(BatchDev bd, InjectArgs a) {
+  __shared__ InjectTile T;
+  const int j = blockIdx.z;
   const DomInst* d = bd.inst_tab + bd.inst[j];
-  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= d->nsites) return;
+  const long long l0 = (long long)blockIdx.x * INJ_SITES, l = l0 + threadIdx.x;
+  const int n = (int)min((long long)INJ_SITES, d->nsites - l0);
+  if (n <= 0) return;
   int dims[4] = {d->dims[0], d->dims[1], d->dims[2], d->dims[3]};
-  int x[4];
+  int x[4], g[4];
   site_coords(l, dims, x);
-  int g[4];
   for (int m = 0; m < 4; ++m) g[m] = (d->origin[m] + x[m]) % a.L[m];
   const int gx = glob_index(g, a.L);
-  double2 acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = make_double2(0.0, 0.0);
-  for (int dir = 0; dir < 8; ++dir) {
+  inject_tile(T, n, a, [&](int dir, int& q, int& ls) -> bool {
     const int mu = dir & 3, step = dir < 4 ? 1 : -1;
     const int y = x[mu] + step;
-    if (y >= 0 && y < dims[mu]) continue;           // hop stays inside the box
-    if (dims[mu] == a.L[mu]) continue;              // box wraps (direction not decomposed)
+    if (y >= 0 && y < dims[mu]) return false;         // hop stays inside the box
+    if (dims[mu] == a.L[mu]) return false;            // box wraps (direction not decomposed)
     int gy[4] = {g[0], g[1], g[2], g[3]};
     gy[mu] = (g[mu] + step + a.L[mu]) % a.L[mu];
-    add_exterior_hop(acc, dir, gx, glob_index(gy, a.L), a, f);
-  }
-  double2* out = a.src + bd.uoff[sys] + 12 * l;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) out[k] = make_double2(-a.kappa * acc[k].x, -a.kappa * acc[k].y);
+    const int yg = glob_index(gy, a.L);
+    q = a.dpi_pos[yg];
+    ls = step > 0 ? gx : yg;
+    return q >= 0;         // always, for a valid geometry (exterior sites lie on dPi)
+  }, [&](int f) { return a.src + bd.uoff[j * a.n_f + f] + 12 * l0; });
 }
 
 // Sources for the frame: t(x) = D_{Lambda1, dLambda0} chi, x in Lambda1 (field order).
-__global__ void k_inject_frame(const int* __restrict__ l1_glob, int n_l1,
-                               const unsigned char* __restrict__ in_l1, InjectArgs a) {
-  const int f = blockIdx.y;
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n_l1) return;
-  const int gx = l1_glob[k];
+__global__ void __launch_bounds__(INJ_SITES) k_inject_frame(const int* __restrict__ l1_glob, int n_l1,
+                                                            const unsigned char* __restrict__ in_l1, InjectArgs a) {
+  __shared__ InjectTile T;
+  const long long k0 = (long long)blockIdx.x * INJ_SITES;
+  const int n = (int)min((long long)INJ_SITES, n_l1 - k0);
+  if (n <= 0) return;
+  const int gx = l1_glob[k0 + min((int)threadIdx.x, n - 1)];
   int g[4];
   site_coords(gx, a.L, g);
-  double2 acc[12];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) acc[c] = make_double2(0.0, 0.0);
-  for (int dir = 0; dir < 8; ++dir) {
+  inject_tile(T, n, a, [&](int dir, int& q, int& ls) -> bool {
     const int mu = dir & 3, step = dir < 4 ? 1 : -1;
     int gy[4] = {g[0], g[1], g[2], g[3]};
     gy[mu] = (g[mu] + step + a.L[mu]) % a.L[mu];
     const int y = glob_index(gy, a.L);
-    if (in_l1[y]) continue;                           // neighbour inside the frame
-    add_exterior_hop(acc, dir, gx, y, a, f);
-  }
-  double2* out = a.src + ((long long)f * n_l1 + k) * 12;
-#pragma unroll
-  for (int c = 0; c < 12; ++c) out[c] = make_double2(-a.kappa * acc[c].x, -a.kappa * acc[c].y);
+    if (in_l1[y]) return false;                       // neighbour inside the frame
+    q = a.dpi_pos[y];
+    ls = step > 0 ? gx : y;
+    return q >= 0;
+  }, [&](int f) { return a.src + ((long long)f * n_l1 + k0) * 12; });
 }
 
 // Sources of the frame pieces: t(x) = D_{Phi1^b, dLambda0^b} chi for x in
 // Phi1^b, the hops into x from the boundary sites of its own core b (batch
 // position j holds Phi1^b, b = blk_of_pos[j], or b = j without the map).
-// grid: (ceil(max_sites/128), n_f, nb)
-__global__ void k_inject_phi(BatchDev bd, InjectArgs a, const int* __restrict__ dpi_kind,
-                             const int* __restrict__ blk_of_pos) {
-  const int f = blockIdx.y, j = blockIdx.z;
-  const int sys = j * a.n_f + f;
+__global__ void __launch_bounds__(INJ_SITES) k_inject_phi(BatchDev bd, InjectArgs a, const int* __restrict__ dpi_kind,
+                                                          const int* __restrict__ blk_of_pos) {
+  __shared__ InjectTile T;
+  const int j = blockIdx.z;
   const int blk = blk_of_pos ? blk_of_pos[j] : j;
   const DomInst* d = bd.inst_tab + bd.inst[j];
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= d->nsites) return;
-  const int gx = d->glob[k];
+  const int f0 = blockIdx.x * INJ_SITES;              // field positions
+  const int n = min(INJ_SITES, d->nsites - f0);
+  if (n <= 0) return;
+  const int v = d->ifm[f0 + min((int)threadIdx.x, n - 1)];
+  const int gx = d->glob[(v >> 30 ? d->n[0] : 0) + (v & ((1 << 30) - 1))];
   int g[4];
   site_coords(gx, a.L, g);
-  double2 acc[12];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) acc[c] = make_double2(0.0, 0.0);
-  for (int dir = 0; dir < 8; ++dir) {
+  inject_tile(T, n, a, [&](int dir, int& q, int& ls) -> bool {
     const int mu = dir & 3, step = dir < 4 ? 1 : -1;
     int gy[4] = {g[0], g[1], g[2], g[3]};
     gy[mu] = (g[mu] + step + a.L[mu]) % a.L[mu];
     const int y = glob_index(gy, a.L);
-    const int q = a.dpi_pos[y];
-    if (q < 0 || dpi_kind[q] != blk) continue;        // not a boundary site of this core
-    add_exterior_hop(acc, dir, gx, y, a, f);
-  }
-  double2* out = a.src + bd.uoff[sys] + 12LL * d->fmap[k];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) out[c] = make_double2(-a.kappa * acc[c].x, -a.kappa * acc[c].y);
+    q = a.dpi_pos[y];
+    ls = step > 0 ? gx : y;
+    return q >= 0 && dpi_kind[q] == blk;              // a boundary site of this core
+  }, [&](int f) { return a.src + bd.uoff[j * a.n_f + f] + 12LL * f0; });
 }
 
 // On every dPi1 site x and field f: q = (Q chi)(x), the sum of the frame-piece
@@ -637,14 +734,14 @@ static dd_status frame_stage(dd_ctx* c, WPlan& P, int n_f, const double* chi, do
   a.kappa = c->kappa;
   a.src = (double2*)src_a;
   BatchDev bd = batch_view(c, *ab);
-  dim3 g1((P.max_phi + 127) / 128, n_f, nb);
-  DD_COUNT_LAUNCH(), k_inject_phi<<<g1, 128, 0, s>>>(bd, a, c->d_dpi_kind, nullptr);
+  const dim3 g1 = inject_grid(c, P.max_phi, n_f, nb);
+  DD_COUNT_LAUNCH(), k_inject_phi<<<g1, INJ_SITES, 0, s>>>(bd, a, c->d_dpi_kind, nullptr);
   if (with_frame) {
     long long phi_user = 0;
     for (int b = 0; b < nb; ++b) phi_user += 12LL * c->inst[c->phi0 + b].d.nsites * n_f;
     a.src = (double2*)src_a + phi_user;
-    dim3 g2((P.n_l1 + 127) / 128, n_f);
-    DD_COUNT_LAUNCH(), k_inject_frame<<<g2, 128, 0, s>>>(P.d_l1_glob, P.n_l1, P.d_in_l1, a);
+    const dim3 g2 = inject_grid(c, P.n_l1, n_f, 1);
+    DD_COUNT_LAUNCH(), k_inject_frame<<<g2, INJ_SITES, 0, s>>>(P.d_l1_glob, P.n_l1, P.d_in_l1, a);
   }
   DD_CUDA(c, cudaGetLastError());
   dd_status r = solve_batch(c, *ab, (const double*)src_a, (double*)sol_a, prm, st, s, true);
@@ -755,8 +852,8 @@ static dd_status apply_w_dev(dd_ctx* c, int n_f, const double* chi, double* wchi
   a.kappa = c->kappa;
   a.src = (double2*)src_o;
   BatchDev bd = batch_view(c, *ob);
-  dim3 g1((c->info.max_omega + 127) / 128, n_f, nb);
-  DD_COUNT_LAUNCH(), k_inject_omega<<<g1, 128, 0, s>>>(bd, a);
+  const dim3 g1 = inject_grid(c, c->info.max_omega, n_f, nb);
+  DD_COUNT_LAUNCH(), k_inject_omega<<<g1, INJ_SITES, 0, s>>>(bd, a);
   DD_CUDA(c, cudaGetLastError());
   dd_solve_stats sb{};
   dd_status rb = solve_batch(c, *ob, (const double*)src_o, (double*)sol_o, prm, &sb, s, true);
@@ -832,14 +929,14 @@ static dd_status apply_w_part_dev(dd_ctx* c, int part, int n_f, const int* ids, 
   a.src = (double2*)src;
   BatchDev bd = batch_view(c, *bt);
   if (part == DD_W_FRAME_Q) {
-    dim3 g1((P.max_phi + 127) / 128, n_f, nblk);
-    DD_COUNT_LAUNCH(), k_inject_phi<<<g1, 128, 0, s>>>(bd, a, c->d_dpi_kind, d_blk);
+    const dim3 g1 = inject_grid(c, P.max_phi, n_f, nblk);
+    DD_COUNT_LAUNCH(), k_inject_phi<<<g1, INJ_SITES, 0, s>>>(bd, a, c->d_dpi_kind, d_blk);
   } else if (part == DD_W_BLOCKS) {
-    dim3 g1((c->info.max_omega + 127) / 128, n_f, nblk);
-    DD_COUNT_LAUNCH(), k_inject_omega<<<g1, 128, 0, s>>>(bd, a);
+    const dim3 g1 = inject_grid(c, c->info.max_omega, n_f, nblk);
+    DD_COUNT_LAUNCH(), k_inject_omega<<<g1, INJ_SITES, 0, s>>>(bd, a);
   } else {
-    dim3 g2((P.n_l1 + 127) / 128, n_f);
-    DD_COUNT_LAUNCH(), k_inject_frame<<<g2, 128, 0, s>>>(P.d_l1_glob, P.n_l1, P.d_in_l1, a);
+    const dim3 g2 = inject_grid(c, P.n_l1, n_f, 1);
+    DD_COUNT_LAUNCH(), k_inject_frame<<<g2, INJ_SITES, 0, s>>>(P.d_l1_glob, P.n_l1, P.d_in_l1, a);
   }
   DD_CUDA(c, cudaGetLastError());
   dd_solve_stats st{};
@@ -1309,8 +1406,8 @@ static dd_status mb_force_dev(dd_ctx* c, int n_f, const double* u, const double*
   a.kappa = c->kappa;
   a.src = (double2*)vsrc;
   BatchDev bd = batch_view(c, *ob);
-  dim3 g1((c->info.max_omega + 127) / 128, n_f, nb);
-  DD_COUNT_LAUNCH(), k_inject_omega<<<g1, 128, 0, s>>>(bd, a);
+  const dim3 g1 = inject_grid(c, c->info.max_omega, n_f, nb);
+  DD_COUNT_LAUNCH(), k_inject_omega<<<g1, INJ_SITES, 0, s>>>(bd, a);
   DD_CUDA(c, cudaGetLastError());
   dd_status r1 = solve_batch(c, *ob, (const double*)vsrc, (double*)vy, prm, &st1, s, true);
   if (r1 == DD_ENOCONV) *noconv = true;
