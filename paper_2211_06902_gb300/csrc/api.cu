@@ -216,13 +216,16 @@ dd_status dd_apply_D_block(dd_ctx* c, dd_domain kind, const int* ids, int nblk, 
     se = ae;
     so = ao;
   }
+  const bool direct = hop_writes_user(c, *b, prec);
   HopArgs h{};
+  h.user = direct ? (double2*)sg.out : nullptr;
   h.p_out = 0; h.in = vo; h.out = oe; h.s1 = se; h.a1 = 1.0; h.b = -c->kappa;
   if ((e = launch_hop(c, *b, prec, h, s)) != DD_OK) return e;
   HopArgs g{};
+  g.user = h.user;
   g.p_out = 1; g.in = ve; g.out = oo; g.s1 = so; g.a1 = 1.0; g.b = -c->kappa;
   if ((e = launch_hop(c, *b, prec, g, s)) != DD_OK) return e;
-  if ((e = launch_unpack(c, *b, oe, oo, sg.out, prec, s)) != DD_OK) return e;
+  if (!direct && (e = launch_unpack(c, *b, oe, oo, sg.out, prec, s)) != DD_OK) return e;
   if ((e = unstage(c, out, ub, sg, s)) != DD_OK) return e;
   // host buffers: the call has synchronised anyway, so report a bounded wait
   // that gave up (device buffers leave it to the next synchronous call)

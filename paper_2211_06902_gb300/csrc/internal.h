@@ -273,7 +273,9 @@ struct HopArgs {
   int lb_fault;             // test hook of the bundle form (dd_debug_wait_fault): CTA 0 leaves
                             // one quarter's bulk copy unissued and waits a few microseconds
   int* queue;               // work-queue counter of the persistent bundle form
+  double2* user;            // output in the caller layout instead of `out` (see hop_writes_user), or null
 };
+bool hop_writes_user(const dd_ctx* c, const Batch& b, dd_prec prec);
 dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a, cudaStream_t s);
 void ensure_nsm(dd_ctx* c);      // c->nsm = SMs of the device
 int hop_variant_count(dd_prec prec);

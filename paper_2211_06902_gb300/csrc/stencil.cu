@@ -83,9 +83,11 @@ __device__ __forceinline__ void hop_one(C (&acc)[12], int n0, int p, int i, int 
 // grid: nitems[p] * nrhs CTAs, rhs fastest (the CTAs that share a site chunk,
 // and so its links, run together and hit L2); one output site per thread.
 // One CTA work unit t = item * nrhs + rhs of the hop launch.
-template <class S, bool CLOV, bool ROWS = false>
+// s0: first site of this CTA within the item; USER: the output goes to the caller layout (a.user)
+// through `stage`, 5 numbers a thread
+template <class S, bool CLOV, bool ROWS = false, bool USER = false>
 __device__ __forceinline__ void hop_unit(const BatchDev& bd, const HopArgs& a, long long t,
-                                         double* red) {
+                                         double* red, int s0 = 0, double2* stage = nullptr) {
   typedef typename StoreTraits<S>::C C;
   typedef typename StoreTraits<S>::T T;
   const int p = a.p_out;
@@ -94,12 +96,14 @@ __device__ __forceinline__ void hop_unit(const BatchDev& bd, const HopArgs& a, l
   const int4 it = (p ? bd.items[1] : bd.items[0])[item];
   const int sys = it.x * bd.nrhs + r;
   if (a.active && !a.active[(long long)sys * a.active_stride]) return;
-  if (a.work_bytes && threadIdx.x == 0) atomicAdd(a.work_bytes, a.site_bytes * it.z);
+  const int cnt = min((int)blockDim.x, it.z - s0);     // sites of this CTA
+  if (cnt <= 0) return;
+  if (a.work_bytes && threadIdx.x == 0) atomicAdd(a.work_bytes, a.site_bytes * cnt);
   const DomInst* dp = bd.inst_tab + bd.inst[it.x];
   const int n0 = dp->n[0];
   const int n_out = p ? dp->n[1] : n0, n_in = p ? n0 : dp->n[1];
-  const int i = it.y + threadIdx.x;
-  const bool live = threadIdx.x < it.z;
+  const int i = it.y + s0 + threadIdx.x;
+  const bool live = (int)threadIdx.x < cnt;
   const S* in_sys = (const S*)a.in + (p ? bd.off[0] : bd.off[1])[sys];
   S* out_sys = (S*)a.out + (p ? bd.off[1] : bd.off[0])[sys];
   C out[12];
@@ -144,7 +148,31 @@ __device__ __forceinline__ void hop_unit(const BatchDev& bd, const HopArgs& a, l
 #pragma unroll
       for (int k = 0; k < 12; ++k) axpy(out[k], a2, v[k]);
     }
-    st_site<12>(out_sys, n_out, i, out);
+    if constexpr (!USER) st_site<12>(out_sys, n_out, i, out);
+  }
+  if constexpr (USER) {
+    // four numbers of each of the warp's sites at a time: whole 64-byte runs, little shared
+    // memory (with all twelve staged it took the L1 that holds the links: 1200 us a call for
+    // 24^4 x 12 rhs)
+    const int lane = threadIdx.x & 31, sites = min(32, cnt - (int)(threadIdx.x & ~31u));
+    double2* mine = stage + (threadIdx.x >> 5) * 32 * 5;
+    const int f = live ? __ldg(dp->fmap + (p ? n0 : 0) + i) : 0;
+    double2* dst = a.user + bd.uoff[sys];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (live)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mine[lane * 5 + k] = to_d2(out[4 * c + k]);
+      __syncwarp();
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int site = e * 8 + (lane >> 2);
+        const int fs = __shfl_sync(0xffffffffu, f, site);
+        if (site < sites) dst[12LL * fs + 4 * c + (lane & 3)] = mine[site * 5 + (lane & 3)];
+      }
+      __syncwarp();
+    }
+    return;
   }
   if constexpr (std::is_same<C, dfc>::value) {
     // the double-float residual kernel: optionally |out|^2 (high parts, FP32 per
@@ -628,6 +656,19 @@ __global__ void __launch_bounds__(HOP_THREADS, MINB) k_hop(BatchDev bd, HopArgs 
     if constexpr (R == 1) hop_unit<S, CLOV, ROWS>(bd, a, blockIdx.x, red);
     else hop_unit_r<S, R>(bd, a, blockIdx.x, red);
   }
+}
+
+// The plain form on TH of an item's 128 sites per CTA, without inner products.  FP64 is bound by
+// the FP64 pipes (about 750 instructions a site, 17 cycles a warp), so the CTAs have to cover all
+// SMs evenly: 16 blocks of 5^4 with one rhs are 48 items, which kept 48 SMs busy for 27 us a hop.
+// USER: the output leaves in the caller layout, which saves dd_apply_D_block a pass over it.
+template <class S, int TH, bool USER>
+__global__ void __launch_bounds__(TH, (std::is_same<S, double2>::value ? 3 : 6) * HOP_THREADS / TH)
+    k_hop_part(BatchDev bd, HopArgs a) {
+  constexpr int PARTS = HOP_THREADS / TH;
+  __shared__ double2 stage[USER ? TH * 5 : 1];
+  hop_unit<S, std::is_same<S, double2>::value, false, USER>(bd, a, blockIdx.x / PARTS, nullptr,
+                                                            (blockIdx.x % PARTS) * TH, stage);
 }
 
 // ---- bundle form: links and neighbour indices by bulk copy ----------------------
@@ -1199,6 +1240,24 @@ static void launch_split(const BatchDev& bd, const HopArgs& a, long long nitems_
   DD_COUNT_LAUNCH(), k_hop_split<S, MINB, PERSIST><<<(unsigned)grid, 2 * HOP_THREADS, 0, s>>>(bd, a, nunits);
 }
 
+template <class S, bool USER>
+static void launch_part(const BatchDev& bd, const HopArgs& a, long long nunits, bool fine, cudaStream_t s) {
+  if (fine) DD_COUNT_LAUNCH(), k_hop_part<S, 32, USER><<<(unsigned)(4 * nunits), 32, 0, s>>>(bd, a);
+  else DD_COUNT_LAUNCH(), k_hop_part<S, HOP_THREADS, USER><<<(unsigned)nunits, HOP_THREADS, 0, s>>>(bd, a);
+}
+
+// The plain form by parts of an item.  PART_UNITS: up to that many (item, rhs) units per SM the
+// CTAs take 32 sites, so that no SM is left with a whole item more than the others.
+constexpr int PART_UNITS = 16;
+static void launch_parts(dd_prec prec, const BatchDev& bd, const HopArgs& a, long long ni, int nsm, cudaStream_t s) {
+  const long long nunits = ni * bd.nrhs;
+  const bool fine = nunits <= (long long)PART_UNITS * nsm;
+  if (!a.user) launch_part<double2, false>(bd, a, nunits, fine, s);
+  else if (prec == DD_F64) launch_part<double2, true>(bd, a, nunits, fine, s);
+  else if (prec == DD_F32) launch_part<float2, true>(bd, a, nunits, fine, s);
+  else launch_part<__nv_bfloat162, true>(bd, a, nunits, fine, s);
+}
+
 static void dispatch_hop(dd_prec prec, int v, const BatchDev& bd, const HopArgs& a, long long ni,
                          int nsm, cudaStream_t s) {
   if (prec == DD_DF64) {
@@ -1296,6 +1355,13 @@ void ensure_nsm(dd_ctx* c) {
   if (c->nsm <= 0) c->nsm = 1;
 }
 
+// Whether the stencil of this batch can write the caller layout itself (HopArgs::user): in the
+// plain form, where no launch variant was tuned or chosen for it.
+bool hop_writes_user(const dd_ctx* c, const Batch& b, dd_prec prec) {
+  const int pi = prec == DD_F64 ? 0 : (prec == DD_F32 ? 1 : 2);
+  return c->forced_variant[pi] < 0 && (!b.tuned[pi] || b.hop_variant[pi] == 0);
+}
+
 dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a0, cudaStream_t s) {
   dd_status st = sync_instances(c);
   if (st != DD_OK) return st;
@@ -1324,13 +1390,19 @@ dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a0,
     rec.which = (prec == DD_F64 || prec == DD_DF64) ? 0 : (prec == DD_F32 ? 1 : 2);
     rec.bytes = 0.0;
     a.work_bytes = c->d_tbytes + rec.which;
-    a.site_bytes = hop_site_bytes(b, prec_bytes(prec), (a.s1 ? 1 : 0) + (a.s2 ? 1 : 0));
+    a.site_bytes = hop_site_bytes(b, prec_bytes(prec), (a.s1 ? 1 : 0) + (a.s2 ? 1 : 0)) +
+                   (a.user ? 192.0 - 12.0 * prec_bytes(prec) : 0.0);
     cudaEventRecord(rec.a, s);
   }
   ensure_nsm(c);
   const int pi = (prec == DD_F64 || prec == DD_DF64) ? 0 : (prec == DD_F32 ? 1 : 2);
   const int v = c->forced_variant[pi] >= 0 ? c->forced_variant[pi] : b.hop_variant[pi];
-  dispatch_hop(prec, v, bd, a, b.nitems[p], c->nsm, s);
+  const bool dots = a.dotq || a.dots || a.dotqs;
+  if (a.user || (prec == DD_F64 && v == 0 && c->forced_variant[0] < 0 && !dots &&
+                 nblk <= (long long)PART_UNITS * c->nsm))
+    launch_parts(prec, bd, a, b.nitems[p], c->nsm, s);
+  else
+    dispatch_hop(prec, v, bd, a, b.nitems[p], c->nsm, s);
   if (tm) {
     cudaEventRecord(rec.b, s);
     c->trec.push_back(rec);
