@@ -591,6 +591,7 @@ dd_status make_batch(dd_ctx* c, const std::vector<int>& inst, int nrhs, Batch& b
   }
   b.nfitems = (int)fitems.size();
   b.user_tot = utot;
+  b.hop_variant[1] = hop_default_f32(b.tot[0] / 12, nrhs);
   dd_status st;
   if ((st = dalloc(c, (void**)&b.d_fitems, sizeof(int4) * std::max<size_t>(1, fitems.size()))) != DD_OK)
     return st;

@@ -94,7 +94,7 @@ struct Batch {
   int nfitems = 0;                          // field order (caller layout), both parities together
   std::vector<int> item_begin[2];
   int maxn[2] = {0, 0};
-  // tuned hop launch variant per precision (f64, f32, bf16) and CUDA graphs of
+  // hop launch variant per precision (f64, f32, bf16; defaults, or tuned) and CUDA graphs of
   // the inner Krylov iterations (krylov.cu), owned by the batch
   mutable int hop_variant[3] = {0, 0, 0};
   mutable bool tuned[3] = {false, false, false};
@@ -279,6 +279,7 @@ bool hop_writes_user(const dd_ctx* c, const Batch& b, dd_prec prec);
 dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a, cudaStream_t s);
 void ensure_nsm(dd_ctx* c);      // c->nsm = SMs of the device
 int hop_variant_count(dd_prec prec);
+int hop_default_f32(long long even_site_rhs, int nrhs);
 // sets the shared-memory attributes of the bundle kernels on the current device
 void hop_bundle_prepare();
 // reads and clears the device error word: DD_ETIMEOUT if a bounded wait gave up

@@ -1215,6 +1215,17 @@ static const HopVariant kVariants16[] = {{5, false, 1}, {4, false, 1}, {8, false
 
 int hop_variant_count(dd_prec prec) { return prec == DD_F64 ? 5 : (prec == DD_F32 ? 22 : 15); }
 
+// The FP32 variant of a batch before any tuning.  The bundle forms share a chunk's links between
+// the rhs of a CTA; they pay off with at least six of them, and from about 1.2 million even sites
+// x rhs on, where the CTAs' start-up no longer shows (FP32 solves, plain / bundle form, ms: 24^4 x
+// 12 rhs 51.2 / 48.4 and x 8 35.8 / 34.8 and x 6 28.1 / 27.7, but x 4 20.3 / 21.4; 20^4 x 12
+// 27.3 / 26.7; 16^4 x 12 12.8 / 13.1).  Whole items of 12 rhs fill a CTA, fewer run better by halves.
+int hop_default_f32(long long even_site_rhs, int nrhs) {
+  const int ngroups = (nrhs + LB_MAX_RHS - 1) / LB_MAX_RHS, rb = (nrhs + ngroups - 1) / ngroups;
+  if (even_site_rhs < 1200000 || rb < 6) return 0;
+  return rb >= 10 ? 13 : 17;
+}
+
 static const HopVariant& variant_of(dd_prec prec, int v) {
   const HopVariant* t = prec == DD_F64 ? kVariants64 : (prec == DD_F32 ? kVariants32 : kVariants16);
   if (v < 0 || v >= hop_variant_count(prec)) v = 0;
