@@ -149,15 +149,15 @@ __device__ __forceinline__ void st_pair(df2s* p, dfc a, dfc b) {
 }
 // (st_pair renormalises through stc)
 __device__ __forceinline__ float2 split_d(double x) {
-  const float h = (float)x;
-  return make_float2(h, (float)(x - (double)h));
+  const float h = narrow(x);
+  return make_float2(h, narrow(x - widen(h)));
 }
 template <> __device__ __forceinline__ dfc cmk<dfc>(double re, double im) {
   const float2 r = split_d(re), i = split_d(im);
   return dfc{make_float2(r.x, i.x), make_float2(r.y, i.y)};
 }
 __device__ __forceinline__ double2 to_d2(dfc a) {
-  return make_double2((double)a.h.x + (double)a.l.x, (double)a.h.y + (double)a.l.y);
+  return make_double2(widen(a.h.x) + widen(a.l.x), widen(a.h.y) + widen(a.l.y));
 }
 __device__ __forceinline__ dfc cadd(dfc a, dfc b) {
   f2p h = pk(a.h), l = pk(a.l);

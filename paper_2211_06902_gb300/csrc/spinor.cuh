@@ -322,7 +322,26 @@ __device__ __forceinline__ void axpy(double2& o, double s, double2 v) {
   o.x = fma(s, v.x, o.x);
   o.y = fma(s, v.y, o.y);
 }
-__device__ __forceinline__ double2 to_d2(float2 a) { return make_double2(a.x, a.y); }
+// float <-> double by integer arithmetic.  A conversion instruction runs on the FP64 pipe (about
+// 1.8 lanes a clock and SM), which bounded the passes between FP32 or double-float vectors and the
+// caller layout: 24 numbers a site, one conversion each and three with the low parts.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (m - 1u < 0x007fffffu || m >= 0x7f800000u) return (double)v;      // denormal, infinite, NaN
+  return m ? __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29))
+           : __hiloint2double((int)b, 0);
+}
+// nearest float (ties to even), as the conversion instruction rounds
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);              // +0, -0
+  if (((hi >> 20) & 0x7ffu) - 897u >= 253u) return (float)x;           // denormal or too large for a float, NaN
+  unsigned m = (((hi & 0x7fffffffu) << 3) | (lo >> 29)) - (896u << 23);
+  const unsigned rem = lo << 3;
+  m += rem > 0x80000000u || (rem == 0x80000000u && (m & 1u)) ? 1u : 0u;
+  return __uint_as_float(m | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double2 to_d2(float2 a) { return make_double2(widen(a.x), widen(a.y)); }
 __device__ __forceinline__ double2 to_d2(double2 a) { return a; }
 // |a|^2 of one component as float (norms for convergence tests)
 __device__ __forceinline__ float nrm2f(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
