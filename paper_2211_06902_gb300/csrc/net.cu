@@ -478,31 +478,44 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         partial[((long long)blockIdx.x * 9 + td) * COUT * CIN + (c2 + c) * CIN + p2 + q] = acc[c][q];
 }
 
-// sum of the per-unit partials (fixed order, FP64): G[k] for k < n.  A CTA sums 32 neighbouring
-// outputs, each warp every 32nd unit (one 256-byte row per load), then the 32 subtotals in order.
-// Bound by HBM (the partials once); one thread per output walking all units took 760 us a layer on
-// average for the 3328 units of 16^4 with 4 rhs, this 123 us.
+// sum of the per-unit partials (fixed order, FP64): G[k] for k < n.  A CTA sums 8 neighbouring
+// outputs (64-byte rows), 128 threads per output every 128th unit, then the subtotals by
+// butterflies.  Bound by the FP64 pipe (two sums a partial; widen() keeps the conversions off
+// it), so the CTAs have to cover the SMs: with 32 outputs a CTA a 16 -> 16 layer was 72 CTAs,
+// and the four layers took 124 us on average for the 3328 units of 16^4 with 4 rhs.
+constexpr int SP_OUT = 8;
 __global__ void __launch_bounds__(1024) k_sum_partials(const float2* __restrict__ partial, long long nunit, int n,
                                                        double2* G) {
-  __shared__ double2 sub[32][33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int k = blockIdx.x * 32 + lane;
+  __shared__ double2 sub[32][SP_OUT];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = lane % SP_OUT, part = lane / SP_OUT;
+  const int k = blockIdx.x * SP_OUT + o;
+  auto fold = [](double2 v) {             // over the four lanes of an output
+#pragma unroll
+    for (int d = SP_OUT; d < 32; d *= 2) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, d);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, d);
+    }
+    return v;
+  };
   double2 a = make_double2(0.0, 0.0);
   if (k < n)
-    for (long long u = warp; u < nunit; u += 32) {
+    for (long long u = warp * 4 + part; u < nunit; u += 128) {
       const float2 v = partial[u * n + k];
-      a.x += v.x;
-      a.y += v.y;
+      a.x += widen(v.x);
+      a.y += widen(v.y);
     }
-  sub[warp][lane] = a;
+  a = fold(a);
+  if (part == 0) sub[warp][o] = a;
   __syncthreads();
-  if (warp || k >= n) return;
-  a = sub[0][lane];
-  for (int w = 1; w < 32; ++w) {
-    a.x += sub[w][lane].x;
-    a.y += sub[w][lane].y;
+  if (warp) return;
+  a = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    a.x += sub[part * 8 + w][o].x;
+    a.y += sub[part * 8 + w][o].y;
   }
-  G[k] = a;
+  a = fold(a);
+  if (part == 0 && k < n) G[k] = a;
 }
 
 // loss and output gradient: y, x spinor activations (4 channels, FP32);
@@ -751,7 +764,7 @@ static dd_status net_loss_grad(dd_ctx* c, dd_net* n, const Batch& b, const Acts&
     if ((e = launch_wgrad(c, b, bd, 1, cin, cout, A.a[l][0], A.a[l][1], Gr.a[l + 1][0], Gr.a[l + 1][1],
                           part + units0 * nw, s)) != DD_OK)
       return e;
-    DD_COUNT_LAUNCH(), k_sum_partials<<<(nw + 31) / 32, 1024, 0, s>>>(part, units0 + units1, nw, G + n->woff[l]);
+    DD_COUNT_LAUNCH(), k_sum_partials<<<(nw + SP_OUT - 1) / SP_OUT, 1024, 0, s>>>(part, units0 + units1, nw, G + n->woff[l]);
     if (l > 0) {
       const float2* Wa = (const float2*)n->d_wadj + n->woff[l];
       for (int p = 0; p < 2; ++p)
