@@ -9,7 +9,7 @@
 // step instead of eight, the links of a chunk serve the cluster's right-hand sides from
 // registers, and the warps' loads of neighbouring sites meet in L1.  The half spinors are
 // summed through shared memory.  What is left is latency on the smallest batches (8^4 x 4
-// rhs: 19 us an iteration, 68 us launched) and the issue rate on larger ones (about 2000
+// rhs: 19 us an iteration) and the issue rate on larger ones (about 2000
 // warp instructions per step of a group).  Vectors stay in global memory (L2), in the
 // layout and slots of the launched form.  8^4 x 4 rhs whole solve 2222 -> 1069 us, action
 // on 8^4 with 2 fields 4910 -> 2284 us.
@@ -533,13 +533,14 @@ void cluster_prepare() {
 // per SM, in waves of 2 CTAs per SM.  rb and cs are those with the least time by this count
 // (measured against every rb <= 4 and cs in 2, 4, 8 on 8^4 .. 20^4 with 1 .. 12 rhs: within 7 %
 // of the best).  An iteration has four hops and about 12 us of barriers and reductions.
-// The launched form needs about 5 us + work / 9800 us a hop (work: even sites x rhs) and 32 us
+// The launched form needs about 5 us + work / 9800 us a hop (work: even sites x rhs) and 14 us
 // of other launches, and streams from DRAM once the vectors outgrow L2: measured whole solves
-// (launched / one launch, us) 8^4 x 4 rhs 2175 / 1044, 12^4 x 4 2970 / 1948, 16^4 x 1
-// 3126 / 2381, 16^4 x 4 5821 / 4702, 20^4 x 2 8086 / 5854, 24^4 x 1 8325 / 7277; from about
-// 400 thousand even sites x rhs on the two meet (16^4 x 12: 12799 / 12092, 20^4 x 5: 14264 /
-// 14846), so the line lies at 300 thousand.  Not taken with the clover term, per-launch
-// timing, a chosen launch form or the wait test, which concern the launched kernels.
+// (launched / one launch, us) 8^4 x 4 rhs 2233 / 982, 12^4 x 4 2890 / 1918, 16^4 x 1
+// 2704 / 2313, 16^4 x 4 5079 / 4442, 20^4 x 2 6615 / 5843, 24^4 x 1 7583 / 7033, but 8 uneven
+// blocks x 5 4626 / 5032, where the counts are 93 and 107 us an iteration; from about 400
+// thousand even sites x rhs on the two meet, so the line lies at 300 thousand.  Not taken with
+// the clover term, per-launch timing, a chosen launch form or the wait test, which concern the
+// launched kernels.
 ClusterPlan cluster_plan(dd_ctx* c, const Batch& b, dd_prec prec) {
   const ClusterPlan none{0, 0};
   if (prec != DD_F32 && prec != DD_BF16) return none;
@@ -563,7 +564,7 @@ ClusterPlan cluster_plan(dd_ctx* c, const Batch& b, dd_prec prec) {
       }
     }
   }
-  return tbest < 4.0 * (5.0 + work / 9800.0) + 32.0 ? best : none;
+  return tbest < 4.0 * (5.0 + work / 9800.0) + 14.0 ? best : none;
 }
 
 dd_status run_cluster(dd_ctx* c, const Batch& b, dd_prec prec, ClusterPlan plan, const void* rhs, void* x, void* r,
