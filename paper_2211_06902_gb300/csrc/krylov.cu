@@ -233,8 +233,9 @@ __global__ void k_convert(BatchDev bd, int p, SD* y, const SS* __restrict__ x, c
 // outer x += sign * e (e of type S) on parity p, for systems still in the
 // outer loop; the outer vector is FP64 (double2) or double-float (df2s)
 // (with partial: |x|^2 per (item, rhs) into slot 0 afterwards, for every
-// system, updated or not, so the outer check needs no separate norm pass)
-template <class O, class S>
+// system, updated or not, so the outer check needs no separate norm pass);
+// SET: x starts at zero, whatever the memory holds, and is written for every system
+template <class O, class S, bool SET = false>
 __global__ void k_axpy64(BatchDev bd, int p, O* x, const S* __restrict__ e, double sign,
                          const SysState* st, double* partial) {
   typedef typename StoreTraits<S>::C C;
@@ -242,11 +243,16 @@ __global__ void k_axpy64(BatchDev bd, int p, O* x, const S* __restrict__ e, doub
   __shared__ double red[64];
   ELEM_PROLOGUE_P
   const bool upd = live && st[sys].outer_active;
-  if (!partial && !upd) return;
+  if (!SET && !partial && !upd) return;
   double acc[1] = {0.0};
   if (live) {
     CO a[12];
-    ld_site<12>(x + o, n, i, a);
+    if constexpr (SET) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) a[k] = cmk<CO>(0.0, 0.0);
+    } else {
+      ld_site<12>(x + o, n, i, a);
+    }
     if (upd) {
       C v[12];
       ld_site<12>(e + o, n, i, v);
@@ -259,8 +265,8 @@ __global__ void k_axpy64(BatchDev bd, int p, O* x, const S* __restrict__ e, doub
           a[k] = make_double2(fma(sign, (double)v[k].x, a[k].x), fma(sign, (double)v[k].y, a[k].y));
         }
       }
-      st_site<12>(x + o, n, i, a);
     }
+    if (SET || upd) st_site<12>(x + o, n, i, a);
     if (partial) {
       if constexpr (std::is_same<CO, dfc>::value) {
         float t = 0.f;
@@ -838,6 +844,15 @@ void axpy_outer(bool dfo, const BatchDev& bd, dim3 g, int p, void* x, const void
   if (dfo) axpy_outer_t<df2s>(bd, g, p, x, v, sp, sign, st, partial, s);
   else axpy_outer_t<double2>(bd, g, p, x, v, sp, sign, st, partial, s);
 }
+// x = v on parity p (zero for systems out of the outer loop), double-float x
+void set_outer(const BatchDev& bd, dim3 g, int p, void* x, const void* v, dd_prec sp, const SysState* st,
+               cudaStream_t s) {
+  if (sp == DD_F32)
+    DD_COUNT_LAUNCH(), k_axpy64<df2s, float2, true><<<g, 128, 0, s>>>(bd, p, (df2s*)x, (const float2*)v, 1.0, st, nullptr);
+  else
+    DD_COUNT_LAUNCH(), k_axpy64<df2s, __nv_bfloat162, true><<<g, 128, 0, s>>>(bd, p, (df2s*)x, (const __nv_bfloat162*)v,
+                                                                              1.0, st, nullptr);
+}
 void norm2_outer(bool dfo, const BatchDev& bd, dim3 g, int p, const void* v, double* partial,
                  cudaStream_t s) {
   if (dfo) DD_COUNT_LAUNCH(), k_norm2<df2s><<<g, 128, 0, s>>>(bd, p, (const df2s*)v, partial, 0);
@@ -1185,15 +1200,35 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
   cudaEvent_t ev0 = evs.a, ev1 = evs.b;
   cudaEventRecord(ev0, s);
 
+  // The whole solve as one graph launch (mixed forms with BiCGstab inner
+  // solves, once the launch form is tuned): the outer checks and their
+  // decisions run on the device (whole_solve below).
+  const int pi_in = ip == DD_F32 ? 1 : 2;
+  const bool graph_solve = (prm->flags & DD_SOLVE_GRAPH_SOLVE) && !c->timing && dfo &&
+                           !(prm->flags & (DD_SOLVE_FGMRES | DD_SOLVE_NET_PRECOND)) &&
+                           (!(prm->flags & DD_SOLVE_AUTOTUNE) || b.tuned[pi_in]);
+  bool all_omega = true;
+  for (int j = 0; j < b.nb; ++j)
+    if (c->inst[b.inst[j]].d.kind != DD_DOMAIN_OMEGA) all_omega = false;
+  const bool net_start = (prm->flags & DD_SOLVE_NET_GUESS) && c->net && all_omega;
+  // The first cycle of a mixed solve starts from r = b and x = 0, so neither is stored for it: the
+  // inner right-hand side comes from b, x is set to the correction, r is b - D x after it.  (Writing
+  // both with b and reading x back took 1.5 ms of the 32^4 batch's 140.6.)
+  // The whole-solve graph has one body for all cycles, and the network starts elsewhere.
+  bool fresh = dfo && !graph_solve && !net_start;
   // b, r = b and x = 0 in one pass over the caller layout; |b|^2 (= |r|^2)
   // partials by a coalesced pass over the parity vectors
-  if ((e = launch_pack_init(c, b, b_user, be, bo, re, ro, xe, xo, op, s)) != DD_OK) return e;
+  if ((e = fresh ? launch_pack(c, b, b_user, be, bo, op, s)
+                 : launch_pack_init(c, b, b_user, be, bo, re, ro, xe, xo, op, s)) != DD_OK)
+    return e;
   if (clov) {
     // solve (1 - kappa A^{-1} H) x = A^{-1} b: b and r = b preconditioned once
     // (in FP64 arithmetic also for the double-float vectors of the mixed forms)
     if ((e = dfo ? clover_apply_inv_df(c, b, be, bo, s) : clover_apply(c, b, be, bo, true, s)) != DD_OK) return e;
-    DD_CUDA(c, cudaMemcpyAsync(re, be, ne * c64, cudaMemcpyDeviceToDevice, s));
-    if (no > 0) DD_CUDA(c, cudaMemcpyAsync(ro, bo, no * c64, cudaMemcpyDeviceToDevice, s));
+    if (!fresh) {
+      DD_CUDA(c, cudaMemcpyAsync(re, be, ne * c64, cudaMemcpyDeviceToDevice, s));
+      if (no > 0) DD_CUDA(c, cudaMemcpyAsync(ro, bo, no * c64, cudaMemcpyDeviceToDevice, s));
+    }
   }
   norm2_outer(dfo, bd, eg, 0, be, partial, s);
   if (has_odd) norm2_outer(dfo, bd, og, 1, bo, partial_o, s);
@@ -1202,10 +1237,7 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
   bool norms_ready = true;
   // learned initial guess: x = N(b), r = b - D x with D x in FP32 (the first
   // correction cycle is followed by an FP64 residual, which absorbs its rounding)
-  bool all_omega = true;
-  for (int j = 0; j < b.nb; ++j)
-    if (c->inst[b.inst[j]].d.kind != DD_DOMAIN_OMEGA) all_omega = false;
-  if ((prm->flags & DD_SOLVE_NET_GUESS) && c->net && all_omega) {
+  if (net_start) {
     void *ge, *go, *te, *to;
     if ((e = ws_get(c, 28, ne * 8, &ge)) || (e = ws_get(c, 29, no * 8 + 16, &go)) ||
         (e = ws_get(c, 80, ne * 8, &te)) || (e = ws_get(c, 81, no * 8 + 16, &to)))
@@ -1257,8 +1289,8 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
   const void* rin_o = ip != DD_F64 ? rso : ro;
   auto to_inner = [&](cudaStream_t q) -> dd_status {
     if (ip != DD_F64) {
-      convert_outer(dfo, ip, bd, eg, 0, w.s, re, st, q);
-      if (has_odd) convert_outer(dfo, ip, bd, og, 1, rso, ro, st, q);
+      convert_outer(dfo, ip, bd, eg, 0, w.s, fresh ? be : re, st, q);
+      if (has_odd) convert_outer(dfo, ip, bd, og, 1, rso, fresh ? bo : ro, st, q);
     }
     DD_CUDA(c, cudaGetLastError());
     return DD_OK;
@@ -1275,8 +1307,13 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
     h.p_out = 1; h.in = w.x; h.out = eo; h.s1 = rin_o; h.a1 = 1.0; h.b = kap;
     dd_status r = launch_hop(c, b, ip, h, q);
     if (r != DD_OK) return r;
-    axpy_outer(dfo, bd, eg, 0, xe, w.x, ip, 1.0, st, q);
-    if (has_odd) axpy_outer(dfo, bd, og, 1, xo, eo, ip, 1.0, st, q);
+    if (fresh) {
+      set_outer(bd, eg, 0, xe, w.x, ip, st, q);
+      if (has_odd) set_outer(bd, og, 1, xo, eo, ip, st, q);
+    } else {
+      axpy_outer(dfo, bd, eg, 0, xe, w.x, ip, 1.0, st, q);
+      if (has_odd) axpy_outer(dfo, bd, og, 1, xo, eo, ip, 1.0, st, q);
+    }
     DD_CUDA(c, cudaGetLastError());
     return DD_OK;
   };
@@ -1298,13 +1335,6 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
     return DD_OK;
   };
   int cycles = 0;
-  // The whole solve as one graph launch (mixed forms with BiCGstab inner
-  // solves, once the launch form is tuned): the outer checks and their
-  // decisions run on the device (whole_solve below).
-  const int pi_in = ip == DD_F32 ? 1 : 2;
-  const bool graph_solve = (prm->flags & DD_SOLVE_GRAPH_SOLVE) && !c->timing && dfo &&
-                           !(prm->flags & (DD_SOLVE_FGMRES | DD_SOLVE_NET_PRECOND)) &&
-                           (!(prm->flags & DD_SOLVE_AUTOTUNE) || b.tuned[pi_in]);
   if (graph_solve) {
     auto run = [&](auto tag) -> dd_status {
       using S = decltype(tag);
@@ -1373,6 +1403,7 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
                                        floor_frac, prm->maxiter, check_every, use_graph, s, &its, device_loop);
     if (e != DD_OK) return e;
     if ((e = correct_x(s)) != DD_OK) return e;
+    fresh = false;                     // (the first cycle ends with a true residual: cyc == 0)
     if (true_residual) {
       if ((e = true_res(s)) != DD_OK) return e;
       norms_ready = dfo;
@@ -1382,6 +1413,10 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
     }
     last_true = true_residual;
     DD_CUDA(c, cudaGetLastError());
+  }
+  if (fresh) {                         // no cycle was needed: b = 0
+    DD_CUDA(c, cudaMemsetAsync(xe, 0, ne * c64, s));
+    if (no > 0) DD_CUDA(c, cudaMemsetAsync(xo, 0, no * c64, s));
   }
   if ((e = launch_unpack(c, b, xe, xo, x_user, op, s)) != DD_OK) return e;
   cudaEventRecord(ev1, s);
