@@ -108,3 +108,53 @@ def test_new_links_refill_every_copy():
         assert np.array_equal(a, c) and not np.array_equal(a, f)
     old.close()
     new.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+def test_stencil_of_many_units_equals_one_rhs_at_a_time(prec):
+    """Whole items per CTA (more than 16 units per SM) and 32 sites per CTA do the same arithmetic on every site."""
+    L = (4, 4, 4, 4)
+    U, ctx, info, _ = make_case(L, 0.13, 0.4, 9, uniform_cores(L, 1, 1))
+    ids, R = list(range(info["nblocks"])), 176       # 16 blocks x 176 rhs of one item per parity
+    n = len(ctx.geom_sites(dd4d.SET_OMEGA, 0))
+    psi = synth.complex_gaussian(11, synth.TAG_RHS, (len(ids), R, n, 12))
+    out = np.zeros_like(psi)
+    ctx.apply_D_block("omega", ids, R, psi, out, prec)
+    for r in (0, 1, 87, R - 1):
+        one, d = np.ascontiguousarray(psi[:, r:r + 1]), np.zeros((len(ids), 1, n, 12), dtype=np.complex128)
+        ctx.apply_D_block("omega", ids, 1, one, d, prec)
+        assert np.array_equal(d[:, 0], out[:, r])
+    ctx.close()
+
+
+def test_fp32_stencil_converts_as_the_host_does():
+    """At kappa = 0 the FP32 stencil returns its input rounded to FP32 and widened again: ties, denormals, both ends."""
+    L = (4, 4, 4, 4)
+    U, ctx, info, _ = make_case(L, 0.0, 0.3, 1, uniform_cores(L, 1, 1))
+    n = len(ctx.geom_sites(dd4d.SET_OMEGA, 0))
+    rng = np.random.default_rng(5)
+    v = rng.standard_normal(24 * n) * 10.0 ** rng.uniform(-44, 35, 24 * n)
+    v[:9] = 0.0, -0.0, 1 + 2.0 ** -24, 1 + 3 * 2.0 ** -24, 2 - 2.0 ** -25, 2.0 ** -149, 2.0 ** -126, 1e38, -2.0 ** -140
+    psi = v.view(np.complex128).reshape(1, 1, n, 12)
+    out = np.zeros_like(psi)
+    ctx.apply_D_block("omega", [0], 1, psi, out, "f32")
+    assert np.array_equal(out.view(np.float64), psi.view(np.float64).astype(np.float32).astype(np.float64))
+    ctx.close()
+
+
+@pytest.mark.parametrize("inner", ["f32", "bf16"])
+def test_nothing_to_solve_after_a_solve(inner):
+    """b = 0 gives x = 0 whatever the work vectors hold from the solve before."""
+    L = (4, 4, 4, 4)
+    U, ctx, info, _ = make_case(L, 0.13, 0.3, 1, uniform_cores(L, 1, 1))
+    ids, n = list(range(info["nblocks"])), len(ctx.geom_sites(dd4d.SET_OMEGA, 0))
+    b = synth.complex_gaussian(4, synth.TAG_RHS, (len(ids), 2, n, 12))
+    x = np.zeros_like(b)
+    assert ctx.solve_blocks("omega", ids, 2, b, x, dd4d.params(TOL, inner_prec=inner))["status"] == dd4d.DD_OK
+    b[:, 1] = 0                                      # every second system
+    ctx.solve_blocks("omega", ids, 2, b, x, dd4d.params(TOL, inner_prec=inner))
+    assert np.all(x[:, 1] == 0) and np.all(np.abs(x[:, 0]).max(axis=(1, 2)) > 0)
+    x[:] = 1
+    st = ctx.solve_blocks("omega", ids, 2, np.zeros_like(b), x, dd4d.params(TOL, inner_prec=inner))
+    assert st["status"] == dd4d.DD_OK and np.all(x == 0)
+    ctx.close()
