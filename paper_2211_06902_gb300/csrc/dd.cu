@@ -64,7 +64,9 @@ __device__ __forceinline__ int glob_index(const int* x, const int* L) {
 // eight directions each warp ran four or five of them for all its lanes, and looked the
 // neighbours up again for every field.  Here the tile's hops are listed direction by direction
 // once, dense warps take them for each field, forward and backward by the same instructions,
-// into sums in shared memory that leave as whole runs.  24^4 with 12 fields: see the launches.
+// into sums in shared memory that leave as whole runs.  On 24^4 with 12 fields the sources of the
+// blocks took 4.6 ms and those of the frame pieces 2.3 ms; the force call there went from 135.5 to
+// 131.1 ms.
 constexpr int INJ_SITES = 128;
 constexpr int INJ_ROW = 13;               // 12 numbers of a site, padded
 struct InjectTile {

@@ -660,8 +660,9 @@ __global__ void __launch_bounds__(HOP_THREADS, MINB) k_hop(BatchDev bd, HopArgs 
 
 // The plain form on TH of an item's 128 sites per CTA, without inner products.  FP64 is bound by
 // the FP64 pipes (about 750 instructions a site, 17 cycles a warp), so the CTAs have to cover all
-// SMs evenly: 16 blocks of 5^4 with one rhs are 48 items, which kept 48 SMs busy for 27 us a hop.
-// USER: the output leaves in the caller layout, which saves dd_apply_D_block a pass over it.
+// SMs evenly: 16 blocks of 5^4 with one rhs are 48 items, which kept 48 SMs busy for 27 us a hop
+// (FP64 stencil call there 83.1 us, now 73.9).  USER: the output leaves in the caller layout, which
+// saves dd_apply_D_block a pass over it (FP32, 24^4 x 12 rhs: 1201 us a call, now 1060).
 template <class S, int TH, bool USER>
 __global__ void __launch_bounds__(TH, (std::is_same<S, double2>::value ? 3 : 6) * HOP_THREADS / TH)
     k_hop_part(BatchDev bd, HopArgs a) {
@@ -1463,8 +1464,8 @@ __global__ void k_pack(BatchDev bd, const double2* __restrict__ user, S* __restr
 // thread that holds them, every warp store touched 32 half-filled sectors: 820 us for
 // FP32 vectors of 24^4 x 12 rhs (1.84 GB moved).  Here the sites go through shared memory (rows of 13, which
 // spreads the 16-byte stores of 8 lanes over all banks) and leave as 512-byte runs per
-// warp: 345 us for the FP32 vectors. (From double-float vectors the conversion to
-// FP64 is the bound, and the two forms take the same time.)
+// warp: 345 us for the FP32 vectors.  From double-float vectors it was bound by the conversions
+// to FP64 (725 us), which widen() takes off the FP64 pipe.
 template <class S>
 __global__ void __launch_bounds__(128) k_unpack(BatchDev bd, const S* __restrict__ ve, const S* __restrict__ vo,
                                                 double2* __restrict__ user) {
