@@ -274,6 +274,13 @@ dd_status dd_set_hop_variant(dd_ctx* ctx, dd_prec prec, int v);
  * incomplete).  on = 0 restores normal launches; the context stays usable.
  * Host-only, no sync. */
 dd_status dd_debug_wait_fault(dd_ctx* ctx, int on);
+
+/* Test hook of the inner solver's sums (no counterpart in the paper).  For the
+ * first nsys systems of the last solve on the context (not split over chunks):
+ * out[3k] the inner target |r|^2 of the last correction cycle (inner_tol^2 times
+ * the |r|^2 that the inner solve summed at its start, or its floor), out[3k + 1],
+ * out[3k + 2] the last alpha = (r^, r) / (r^, M p).  Host array.  Synchronous. */
+dd_status dd_debug_inner_sums(dd_ctx* ctx, int nsys, double* out);
 int dd_hop_variants(dd_prec prec);
 const char* dd_hop_variant_name(dd_prec prec, int v);
 

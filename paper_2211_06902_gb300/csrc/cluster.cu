@@ -27,10 +27,25 @@ constexpr int CL_THREADS = 512;        // two groups of 8 warps
 constexpr int CL_GROUPS = 2;
 constexpr int CL_R = 4;                // most right-hand sides per cluster
 constexpr int CL_DOTS = 7;
-constexpr int CL_OWN = 192;            // threads of a group that own output pairs (6 warps)
+constexpr int CL_OWN = 192 + 1;        // threads of a group that own output pairs (6 warps), padded
 constexpr int CL_UBUF = 8 * 6 * 32;    // half-spinor numbers of one 32-site chunk and rhs
+// An inner product adds four numbers a lane and step in FP32.  After six steps the lane has added
+// the 24 numbers that a site has in the launched form; the warp's sum of them (768 numbers, as
+// there) is set aside, and everything above is FP64.  A lane has one step on 8^4, seven with framed
+// 9^4 blocks and up to 36 on the largest batches taken; one FP32 sum over all of them was up to 72
+// units of FP32 rounding off where these are at most 30.  A run's end costs a lane about 100
+// instructions (16^4 x 4 rhs 4517 us a solve, without it 4417; 8^4 x 4 rhs has none).
+constexpr int CL_FP32_STEPS = 6;
 constexpr size_t CL_UBYTES = sizeof(float2) * CL_GROUPS * 2 * CL_UBUF;
-constexpr size_t cl_smem_bytes(int rb) { return CL_UBYTES + sizeof(float) * CL_GROUPS * CL_DOTS * rb * CL_OWN; }
+// half spinors, the lanes' sums, the warps' sums of `runs` runs of steps
+constexpr size_t cl_smem_bytes(int rb, int runs) {
+  return CL_UBYTES + sizeof(float) * CL_DOTS * rb * (CL_GROUPS * CL_OWN + CL_THREADS / 32 * runs);
+}
+constexpr int CL_MAX_RUNS = 6;         // (see cluster_plan)
+// runs of a lane with n steps
+__host__ __device__ constexpr int cl_runs(int n) { return (n + CL_FP32_STEPS - 1) / CL_FP32_STEPS; }
+// steps of a lane in a hop: its share of nq chunks
+__host__ __device__ constexpr int cl_steps(int nq, int cs) { return (nq + CL_GROUPS * cs - 1) / (CL_GROUPS * cs); }
 
 struct ClArgs {
   const void* rhs;
@@ -127,6 +142,22 @@ __device__ __forceinline__ const unsigned char* cl_bundle(const DomInst& d) {
   if constexpr (std::is_same<S, float2>::value) return d.lb32;
   else return d.lb16;
 }
+// where a CTA's sum of a warp stands, [run][warp][system][number] (zero between the reductions)
+__device__ __forceinline__ int cl_at(int R, int run, int warp, int rr, int k) {
+  return ((run * (CL_THREADS / 32) + warp) * R + rr) * CL_DOTS + k;
+}
+__device__ __forceinline__ float cl_warp_sum(float v) {           // in lane 0
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+// the same sum of 32 neighbouring numbers in shared memory, with the same tree
+template <int N = 32>
+__device__ __forceinline__ float cl_row_sum(const float* v) {
+  if constexpr (N == 1) return v[0];
+  else return cl_row_sum<N / 2>(v) + cl_row_sum<N / 2>(v + 32 / N);
+}
+
 // MODE 0: out = H in.  MODE 1: out = self - k2 H in with (r^, out).
 // MODE 2: the same with (r^, out), (out, self), |out|^2, (r^, self).
 // Warp w of a group takes direction w of the group's 32 sites, for each active rhs in turn
@@ -134,13 +165,18 @@ __device__ __forceinline__ const unsigned char* cl_bundle(const DomInst& d) {
 // one component pair each.
 template <class S, int MODE>
 __device__ __forceinline__ void cl_hop(const ClView& V, const ClArgs& a, const ClState* st, int p, S* in, S* out,
-                                       S* self, float2* ubuf, float* dacc, unsigned& buf) {
+                                       S* self, float2* ubuf, float* dacc, float* ps, unsigned& buf) {
   const int n_out = V.n[p], n_in = V.n[1 - p];
   const int w = V.w, lane = V.lane;
   constexpr int NK = MODE == 0 ? 0 : (MODE == 1 ? 2 : 7);
-  float* my = dacc + (V.g * CL_DOTS * V.R) * CL_OWN + w * 32 + lane;
-  if (w < 6)
-    for (int k = 0; k < NK * V.R; ++k) my[k * CL_OWN] = 0.f;
+  float* row = dacc + (V.g * CL_DOTS * V.R) * CL_OWN + w * 32;     // number k of system rr at (k R + rr) CL_OWN
+  float* my = row + lane;
+  auto clear = [&]() {
+#pragma unroll
+    for (int k = 0; k < NK * CL_R; ++k)
+      if (k < NK * V.R) my[k * CL_OWN] = 0.f;
+  };
+  if (w < 6) clear();
   const unsigned char* base = cl_bundle<S>(*V.d) + lb_quarter_base(p, V.n[0]) * lb_quarter_bytes<S>();
   const float mk2 = (float)-a.k2;
   // the neighbour index of the next chunk is read one chunk ahead (that of the first one
@@ -148,6 +184,17 @@ __device__ __forceinline__ void cl_hop(const ClView& V, const ClArgs& a, const C
   auto index = [&](int q) {
     return __ldg(reinterpret_cast<const int*>(base + (long long)q * lb_quarter_bytes<S>() + lb_link_bytes<S>()) +
                  w * LB_LANES + lane);
+  };
+  // a run is over: lane (k, rr) adds up its numbers of the warp's lanes
+  int steps = 0, run = 0;
+  auto fold = [&](bool last) {
+    if (w >= 6) return;
+    __syncwarp();
+    if (lane < NK * V.R) ps[cl_at(V.R, run, threadIdx.x >> 5, lane % V.R, lane / V.R)] = cl_row_sum(row + lane * CL_OWN);
+    if (last) return;
+    __syncwarp();
+    clear();
+    ++run;
   };
   int jn = V.j0[p];
   for (int q = V.q0[p]; q < V.q1[p]; ++q) {
@@ -231,33 +278,40 @@ __device__ __forceinline__ void cl_hop(const ClView& V, const ClArgs& a, const C
       }
       st_pair(out + e, o[0], o[1]);
     }
+    if constexpr (MODE > 0)
+      if (++steps == CL_FP32_STEPS && q + 1 < V.q1[p]) {
+        fold(false);
+        steps = 0;
+      }
   }
+  if constexpr (MODE > 0) fold(true);
 }
 
-// sums over the cluster of NK numbers per system: each thread brings val(rr, k); warps in
-// FP32, warps of the CTA and CTAs of the cluster in FP64, in a fixed order (trees of 16 and of
-// the cluster's CTAs: an FP64 addition takes tens of cycles, so their chain is kept short).
-// wpart: CTA scratch; slot: this CTA's sums, read by the others until the cluster barrier after
-// the next one.  On return sums[rr * NK + k] holds the result in every CTA.
-template <int NK, class F>
-__device__ __forceinline__ void cl_reduce(const ClView& V, const ClState* st, double* wpart, double* slot, double* sums,
-                                          F val) {
+// sums over the cluster of NK numbers per system from the warps' sums ps (`runs` of them, zero where
+// a warp has fewer): warps of the CTA and CTAs of the cluster in FP64, in a fixed order (trees of
+// 16 and of the cluster's CTAs: an FP64 addition takes tens of cycles, so their chain is kept
+// short).  slot: this CTA's sums, read by the others until the cluster barrier after the next one.
+// On return sums[rr * NK + k] holds the result in every CTA, and ps is zero again.
+template <int NK>
+__device__ __forceinline__ void cl_reduce(const ClView& V, const ClState* st, float* ps, int runs, double* slot,
+                                          double* sums) {
   constexpr int NW = CL_THREADS / 32;
   const int wi = threadIdx.x >> 5;
-  for (int rr = 0; rr < V.R; ++rr) {
-    if (!st[rr].active) continue;
-#pragma unroll
-    for (int k = 0; k < NK; ++k) {
-      float v = val(rr, k);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (V.lane == 0) wpart[(wi * CL_R + rr) * CL_DOTS + k] = (double)v;
-    }
-  }
   __syncthreads();
   for (int e = wi; e < V.R * NK; e += NW) {
     if (!st[e / NK].active) continue;
-    double v = V.lane < NW ? wpart[(V.lane * CL_R + e / NK) * CL_DOTS + e % NK] : 0.0;
+    double v = 0.0;
+    if (V.lane < NW) {
+      float* at = ps + cl_at(V.R, 0, V.lane, e / NK, e % NK);
+      v = widen(*at);
+      *at = 0.f;
+#pragma unroll 1
+      for (int k = 1; k < runs; ++k) {
+        at += cl_at(V.R, 1, 0, 0, 0);
+        v += widen(*at);
+        *at = 0.f;
+      }
+    }
 #pragma unroll
     for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if (V.lane == 0) slot[e] = v;
@@ -288,7 +342,7 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
   extern __shared__ __align__(16) unsigned char cl_smem[];
   float2* ubuf = reinterpret_cast<float2*>(cl_smem);
   float* dacc = reinterpret_cast<float*>(cl_smem + CL_UBYTES);
-  __shared__ double wpart[CL_THREADS / 32 * CL_R * CL_DOTS];
+  float* ps = dacc + CL_GROUPS * CL_DOTS * a.rb * CL_OWN;
   __shared__ double slots[3][CL_R * CL_DOTS];
   __shared__ double sums[CL_R * CL_DOTS];
   __shared__ ClState st[CL_R];
@@ -328,10 +382,12 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
     at = V.off[rr] + ((long long)(e % 6) * n0 + i) * 2;
     return i < n0;
   };
-  const float* mydot = dacc + (V.g * CL_DOTS * V.R) * CL_OWN + V.w * 32 + V.lane;
-  auto dots = [&](int rr, int k) -> float { return V.w < 6 ? mydot[(k * V.R + rr) * CL_OWN] : 0.f; };
+  // most runs of a warp, in a hop and in a pass over the vectors
+  const int steps = cl_steps((V.n[0] + 31) / 32, (int)nc);
+  const int hruns = cl_runs(steps), vruns = cl_runs((6 * steps + 7) / 8);
   unsigned buf = 0;
 
+  for (int e = threadIdx.x; e < cl_at(V.R, hruns, 0, 0, 0); e += CL_THREADS) ps[e] = 0.f;
   // r = p = rhs, x = 0, (r^, r), |r|^2 and the targets
   if (threadIdx.x < V.R) {
     st[threadIdx.x] = ClState{};
@@ -340,35 +396,44 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
     offs[CL_R + threadIdx.x] = bd.off[1][V.sys0 + threadIdx.x];
   }
   __syncthreads();
-  float part[CL_R][3];
+  const int wi = threadIdx.x >> 5;
+#pragma unroll 1
+  for (int rr = 0; rr < V.R; ++rr) {
+    float part[3] = {0.f, 0.f, 0.f};
+    int run = 0;
+    auto fold = [&]() {
 #pragma unroll
-  for (int rr = 0; rr < CL_R; ++rr) {
-    part[rr][0] = part[rr][1] = part[rr][2] = 0.f;
-    if (rr >= V.R) continue;
-    for (int e = V.w; e < ne; e += 8) {
-      long long at;
-      if (!elem(rr, e, at)) continue;
-      float2 b[2], h[2];
-      ld_pair((const S*)a.rhs + at, b[0], b[1]);
-      st_pair(r + at, b[0], b[1]);
-      st_pair(pv + at, b[0], b[1]);
-      st_pair(x + at, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
-      ld_rhat_pair<S>(a.seed, V.sys0 + rr, (const S*)nullptr, n0, (V.q0[0] + e / 6) * 32 + V.lane, e % 6, h[0], h[1]);
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        part[rr][0] = fmaf(h[k].x, b[k].x, fmaf(h[k].y, b[k].y, part[rr][0]));
-        part[rr][1] = fmaf(h[k].x, b[k].y, fmaf(-h[k].y, b[k].x, part[rr][1]));
-        part[rr][2] = fmaf(b[k].x, b[k].x, fmaf(b[k].y, b[k].y, part[rr][2]));
+      for (int k = 0; k < 3; ++k) {
+        const float v = cl_warp_sum(part[k]);
+        if (V.lane == 0) ps[cl_at(V.R, run, wi, rr, k)] = v;
+        part[k] = 0.f;
       }
-    }
-  }
-  cl_reduce<3>(V, st, wpart, slots[0], sums, [&](int rr, int k) -> float {
-    float o = 0.f;
+      ++run;
+    };
+    int e = V.w;
+#pragma unroll 1
+    do {
+      const int ee = min(ne, e + 8 * CL_FP32_STEPS);
+      for (; e < ee; e += 8) {
+        long long at;
+        if (!elem(rr, e, at)) continue;
+        float2 b[2], h[2];
+        ld_pair((const S*)a.rhs + at, b[0], b[1]);
+        st_pair(r + at, b[0], b[1]);
+        st_pair(pv + at, b[0], b[1]);
+        st_pair(x + at, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+        ld_rhat_pair<S>(a.seed, V.sys0 + rr, (const S*)nullptr, n0, (V.q0[0] + e / 6) * 32 + V.lane, e % 6, h[0], h[1]);
 #pragma unroll
-    for (int q = 0; q < CL_R; ++q)
-      if (q == rr) o = k == 0 ? part[q][0] : (k == 1 ? part[q][1] : part[q][2]);
-    return o;
-  });
+        for (int k = 0; k < 2; ++k) {
+          part[0] = fmaf(h[k].x, b[k].x, fmaf(h[k].y, b[k].y, part[0]));
+          part[1] = fmaf(h[k].x, b[k].y, fmaf(-h[k].y, b[k].x, part[1]));
+          part[2] = fmaf(b[k].x, b[k].x, fmaf(b[k].y, b[k].y, part[2]));
+        }
+      }
+      fold();
+    } while (e < ne);
+  }
+  cl_reduce<3>(V, st, ps, vruns, slots[0], sums);
   if (threadIdx.x < V.R) {
     ClState& z = st[threadIdx.x];
     const SysState& g = a.st[V.sys0 + threadIdx.x];
@@ -387,10 +452,10 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
     bool any = false;
     for (int rr = 0; rr < V.R; ++rr) any = any || st[rr].active;
     if (!any) break;                                  // the same decision in every CTA
-    cl_hop<S, 0>(V, a, st, 1, pv, tmp, (S*)nullptr, ubuf, dacc, buf);
+    cl_hop<S, 0>(V, a, st, 1, pv, tmp, (S*)nullptr, ubuf, dacc, ps, buf);
     cl_sync();
-    cl_hop<S, 1>(V, a, st, 0, tmp, v, pv, ubuf, dacc, buf);
-    cl_reduce<2>(V, st, wpart, slots[0], sums, dots);
+    cl_hop<S, 1>(V, a, st, 0, tmp, v, pv, ubuf, dacc, ps, buf);
+    cl_reduce<2>(V, st, ps, hruns, slots[0], sums);
     if (threadIdx.x < V.R && st[threadIdx.x].active) {
       ClState& z = st[threadIdx.x];
       z.iters += 1;
@@ -418,10 +483,10 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
       }
     }
     cl_sync();
-    cl_hop<S, 0>(V, a, st, 1, s, tmp, (S*)nullptr, ubuf, dacc, buf);
+    cl_hop<S, 0>(V, a, st, 1, s, tmp, (S*)nullptr, ubuf, dacc, ps, buf);
     cl_sync();
-    cl_hop<S, 2>(V, a, st, 0, tmp, t, s, ubuf, dacc, buf);
-    cl_reduce<7>(V, st, wpart, slots[1], sums, dots);
+    cl_hop<S, 2>(V, a, st, 0, tmp, t, s, ubuf, dacc, ps, buf);
+    cl_reduce<7>(V, st, ps, hruns, slots[1], sums);
     if (threadIdx.x < V.R && st[threadIdx.x].active) {
       ClState& z = st[threadIdx.x];
       const double* q = sums + threadIdx.x * 7;       // (r^, t), (t, s), |t|^2, (r^, s)
@@ -440,40 +505,47 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
     // x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v) ; |r|^2
 #pragma unroll
     for (int rr = 0; rr < CL_R; ++rr) {
-      part[rr][0] = 0.f;
       if (rr >= V.R || !st[rr].active) continue;
+      float part = 0.f;
+      int run = 0;
+      auto fold = [&]() {
+        const float v = cl_warp_sum(part);
+        if (V.lane == 0) ps[cl_at(V.R, run, wi, rr, 0)] = v;
+        part = 0.f;
+        ++run;
+      };
       const float2 al = make_float2((float)st[rr].alpha.x, (float)st[rr].alpha.y);
       const float2 om = make_float2((float)st[rr].omega.x, (float)st[rr].omega.y);
       const float2 be = make_float2((float)st[rr].beta.x, (float)st[rr].beta.y);
-      for (int e = V.w; e < ne; e += 8) {
-        long long at;
-        if (!elem(rr, e, at)) continue;
-        float2 xv[2], pp[2], sv[2], tv[2], vv[2];
-        ld_pair(x + at, xv[0], xv[1]);
-        ld_pair(pv + at, pp[0], pp[1]);
-        ld_pair(s + at, sv[0], sv[1]);
-        ld_pair(t + at, tv[0], tv[1]);
-        ld_pair(v + at, vv[0], vv[1]);
+      int e = V.w;
+#pragma unroll 1
+      do {
+        const int ee = min(ne, e + 8 * CL_FP32_STEPS);
+        for (; e < ee; e += 8) {
+          long long at;
+          if (!elem(rr, e, at)) continue;
+          float2 xv[2], pp[2], sv[2], tv[2], vv[2];
+          ld_pair(x + at, xv[0], xv[1]);
+          ld_pair(pv + at, pp[0], pp[1]);
+          ld_pair(s + at, sv[0], sv[1]);
+          ld_pair(t + at, tv[0], tv[1]);
+          ld_pair(v + at, vv[0], vv[1]);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          xv[k] = cadd(xv[k], cadd(cmul(al, pp[k]), cmul(om, sv[k])));
-          const float2 q = csub(sv[k], cmul(om, tv[k]));
-          part[rr][0] = fmaf(q.x, q.x, fmaf(q.y, q.y, part[rr][0]));
-          pp[k] = cadd(q, cmul(be, csub(pp[k], cmul(om, vv[k]))));
-          sv[k] = q;
+          for (int k = 0; k < 2; ++k) {
+            xv[k] = cadd(xv[k], cadd(cmul(al, pp[k]), cmul(om, sv[k])));
+            const float2 q = csub(sv[k], cmul(om, tv[k]));
+            part = fmaf(q.x, q.x, fmaf(q.y, q.y, part));
+            pp[k] = cadd(q, cmul(be, csub(pp[k], cmul(om, vv[k]))));
+            sv[k] = q;
+          }
+          st_pair(x + at, xv[0], xv[1]);
+          st_pair(r + at, sv[0], sv[1]);
+          st_pair(pv + at, pp[0], pp[1]);
         }
-        st_pair(x + at, xv[0], xv[1]);
-        st_pair(r + at, sv[0], sv[1]);
-        st_pair(pv + at, pp[0], pp[1]);
-      }
+        fold();
+      } while (e < ne);
     }
-    cl_reduce<1>(V, st, wpart, slots[2], sums, [&](int rr, int) -> float {
-      float o = 0.f;
-#pragma unroll
-      for (int q = 0; q < CL_R; ++q)
-        if (q == rr) o = part[q][0];
-      return o;
-    });
+    cl_reduce<1>(V, st, ps, vruns, slots[2], sums);
     if (threadIdx.x < V.R && st[threadIdx.x].active) {
       ClState& z = st[threadIdx.x];
       z.rr = sums[threadIdx.x];
@@ -488,6 +560,8 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
     g.rr = z.rr;
     g.target2 = z.target2;
     g.rho = z.rho;
+    g.alpha = z.alpha;
+    g.omega = z.omega;
     g.status = z.status;
     g.iters = z.iters;
     g.active = z.active;
@@ -496,11 +570,11 @@ __global__ void __launch_bounds__(CL_THREADS, 2) k_cl_bicgstab(BatchDev bd, ClAr
 }
 
 template <class S>
-cudaError_t cl_launch(const BatchDev& bd, const ClArgs& a, int clusters, int cs, cudaStream_t s) {
+cudaError_t cl_launch(const BatchDev& bd, const ClArgs& a, int clusters, int cs, int runs, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(clusters * cs));
   cfg.blockDim = dim3(CL_THREADS);
-  cfg.dynamicSmemBytes = cl_smem_bytes(a.rb);
+  cfg.dynamicSmemBytes = cl_smem_bytes(a.rb, runs);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -520,8 +594,8 @@ void cluster_prepare() {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || done[dev]) return;
-  cudaFuncSetAttribute(k_cl_bicgstab<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem_bytes(CL_R));
-  cudaFuncSetAttribute(k_cl_bicgstab<__nv_bfloat162>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem_bytes(CL_R));
+  cudaFuncSetAttribute(k_cl_bicgstab<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem_bytes(CL_R, CL_MAX_RUNS));
+  cudaFuncSetAttribute(k_cl_bicgstab<__nv_bfloat162>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem_bytes(CL_R, CL_MAX_RUNS));
   done[dev] = true;
 }
 
@@ -556,7 +630,8 @@ ClusterPlan cluster_plan(dd_ctx* c, const Batch& b, dd_prec prec) {
     for (int cs = 1; cs <= 8; cs *= 2) {
       const long long ctas = b.nb * ng * cs;
       const double waves = (double)((ctas + 2LL * c->nsm - 1) / (2LL * c->nsm));
-      const double steps = (double)((nq + CL_GROUPS * cs - 1) / (CL_GROUPS * cs)) * rb;
+      if (cl_runs(cl_steps(nq, cs)) > CL_MAX_RUNS) continue;   // 37 steps and more are never the faster form
+      const double steps = (double)cl_steps(nq, cs) * rb;
       const double t = waves * (4.0 * steps * (ctas > c->nsm ? 1.25 : 1.0) + 12.0);
       if (best.cs == 0 || t < tbest) {
         best = {rb, cs};
@@ -584,8 +659,9 @@ dd_status run_cluster(dd_ctx* c, const Batch& b, dd_prec prec, ClusterPlan plan,
   cluster_prepare();
   BatchDev bd = batch_view(c, b);
   DD_COUNT_LAUNCH();
-  const cudaError_t e = prec == DD_F32 ? cl_launch<float2>(bd, a, b.nb * a.ngroups, plan.cs, q)
-                                       : cl_launch<__nv_bfloat162>(bd, a, b.nb * a.ngroups, plan.cs, q);
+  const int clusters = b.nb * a.ngroups, runs = std::max(1, cl_runs(cl_steps((b.maxn[0] + 31) / 32, plan.cs)));
+  const cudaError_t e = prec == DD_F32 ? cl_launch<float2>(bd, a, clusters, plan.cs, runs, q)
+                                       : cl_launch<__nv_bfloat162>(bd, a, clusters, plan.cs, runs, q);
   DD_CUDA(c, e);
   return DD_OK;
 }

@@ -1457,3 +1457,20 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
 }
 
 }  // namespace dd
+
+using namespace dd;
+
+extern "C" dd_status dd_debug_inner_sums(dd_ctx* c, int nsys, double* out) {
+  if (!c || !out || nsys < 1) return DD_EINVAL;
+  auto* ws = reinterpret_cast<Workspace*>(c->scratch);
+  if (nsys > c->last_stats.systems || !ws || ws->bufs.size() <= 16 || ws->sizes[16] < sizeof(SysState) * nsys)
+    return fail(c, DD_EINVAL, "no solve of that many systems before");
+  std::vector<SysState> h(nsys);
+  DD_CUDA(c, cudaMemcpy(h.data(), ws->bufs[16], sizeof(SysState) * nsys, cudaMemcpyDeviceToHost));
+  for (int k = 0; k < nsys; ++k) {
+    out[3 * k] = h[k].target2;
+    out[3 * k + 1] = h[k].alpha.x;
+    out[3 * k + 2] = h[k].alpha.y;
+  }
+  return DD_OK;
+}
