@@ -236,7 +236,9 @@ dd_status dd_geom_block(dd_ctx* ctx, int block, int origin[4], int side[4],
  * ignored for FULL and LAMBDA1, which take nblk = 1) and nrhs fields each.
  * in/out layout: [blk][rhs][site in the domain's field order][12] complex128.
  * prec selects the storage/arithmetic of the stencil (FP64, or FP32 / BF16
- * storage with FP32 arithmetic). */
+ * storage of in and the links with FP32 arithmetic).  The DD_BF16 result is the
+ * FP32 sums, whatever ran on the blocks before; under a launch variant chosen
+ * with dd_set_hop_variant, whose vectors are BF16, it is rounded to BF16. */
 dd_status dd_apply_D_block(dd_ctx* ctx, dd_domain kind, const int* ids, int nblk,
                            int nrhs, const double* in, double* out, dd_prec prec,
                            void* stream);

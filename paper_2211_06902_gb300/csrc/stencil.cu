@@ -1367,11 +1367,14 @@ void ensure_nsm(dd_ctx* c) {
   if (c->nsm <= 0) c->nsm = 1;
 }
 
-// Whether the stencil of this batch can write the caller layout itself (HopArgs::user): in the
-// plain form, where no launch variant was tuned or chosen for it.
+// Whether the stencil of this batch writes the caller layout itself (HopArgs::user): in the plain
+// form, where no launch variant was tuned or chosen for it.  With BF16 storage a tuned variant does
+// not count: its output vectors would round the FP32 sums to BF16, and the call's answer would
+// depend on what ran on the batch before.  (BF16, 24^4 x 12 rhs: 918 us a call, 1044 by the tuned
+// variant and a pass over its output; 8^4 x 1 rhs 27.5 against 25.9.)
 bool hop_writes_user(const dd_ctx* c, const Batch& b, dd_prec prec) {
   const int pi = prec == DD_F64 ? 0 : (prec == DD_F32 ? 1 : 2);
-  return c->forced_variant[pi] < 0 && (!b.tuned[pi] || b.hop_variant[pi] == 0);
+  return c->forced_variant[pi] < 0 && (prec == DD_BF16 || !b.tuned[pi] || b.hop_variant[pi] == 0);
 }
 
 dd_status launch_hop(dd_ctx* c, const Batch& b, dd_prec prec, const HopArgs& a0, cudaStream_t s) {
