@@ -178,7 +178,8 @@ dd_status dd_set_kappa(dd_ctx* ctx, double kappa);
  * at the first mixed solve after A changes.  dd_mb_force, dd_apply_D_block at
  * DD_F32 / DD_BF16, dd_apply_D_block_noalloc and the learned network
  * (DD_SOLVE_NET_GUESS, DD_SOLVE_NET_PRECOND) return DD_EINVAL with the term
- * on.  c_sw = 0 turns it off (the default). */
+ * on.  c_sw = 0 turns it off (the default)
+ * and frees the FP32 copies. */
 dd_status dd_set_clover(dd_ctx* ctx, double c_sw);
 /* c_A = max_x |A_x|_inf * max_x |A_x^{-1}|_inf, the bound of cond_2(A) the solves
  * divide their tolerance by (1 without the term). */
@@ -187,7 +188,11 @@ dd_status dd_clover_cond(dd_ctx* ctx, double* c_A);
 /* Gauge links U_mu(x) in SU(3) (paper Sec. 1).  Host buffer, layout
  * [site (global index)][mu 0..3][3][3] complex128 (row-major 3x3).  The
  * stored links are not modified; the time boundary sign is applied by the
- * operator.  Rebuilds every gathered per-domain copy.  Synchronous. */
+ * operator.  Makes every gathered per-domain copy stale; a copy keeps its
+ * memory and is filled again at its next use.  Copies of a precision that were
+ * not used under the links before are freed (here and in dd_gauge_random; in
+ * dd_md_trajectory those not used during the last eight updates), and all stale
+ * ones when an allocation of the context runs out of memory.  Synchronous. */
 dd_status dd_gauge_upload(dd_ctx* ctx, const double* U_host);
 
 /* Synthetic links drawn on the device (the paper's links U_mu(x) in SU(3),
@@ -276,6 +281,12 @@ dd_status dd_set_hop_variant(dd_ctx* ctx, dd_prec prec, int v);
  * incomplete).  on = 0 restores normal launches; the context stays usable.
  * Host-only, no sync. */
 dd_status dd_debug_wait_fault(dd_ctx* ctx, int on);
+
+/* Test hook of the memory path: the k-th device allocation of the context from
+ * now on (k = 1, 2, ...) acts once as if the device were out of memory; 0 takes
+ * it back.  The allocation then gives back what the context can spare (below,
+ * dd_gauge_upload) and is tried again, or the call returns DD_ENOMEM.  Host-only. */
+dd_status dd_debug_alloc_fault(dd_ctx* ctx, int k);
 
 /* Test hook of the inner solver's sums (no counterpart in the paper).  For the
  * first nsys systems of the last solve on the context (not split over chunks):

@@ -473,6 +473,8 @@ dd_status dd_set_clover(dd_ctx* c, double csw) {
   c->csw = csw;
   if (csw == 0.0) {
     c->clover_ready = false;
+    for (auto& in : c->inst)
+      if (drop_clover_bundles(in)) c->inst_dirty = true;
     return DD_OK;
   }
   return clover_build(c);

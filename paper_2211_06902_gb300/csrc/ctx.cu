@@ -22,31 +22,67 @@ dd_status cuda_fail(dd_ctx* c, cudaError_t e, const char* where) {
   return fail(c, DD_ECUDA, m);
 }
 
-// gives back the link copies that an earlier gauge field left behind; true if there were any
-static bool drop_stale_links(dd_ctx* c) {
+// frees a copy and its pointer in the instance's descriptor
+template <class T>
+static bool drop_copy(void*& buf, const T*& in_table) {
+  in_table = nullptr;
+  if (!buf) return false;
+  dfree(buf);
+  buf = nullptr;
+  return true;
+}
+
+// gives back the link copies of an instance that do not hold the current links and have not been
+// used under the last `unused` gauge fields before; true if there were any.  The device's instance
+// table is not marked for an upload (it may be needed inside a stream capture): nothing reads a
+// copy before ensure_links has filled it, which does mark it.
+static bool drop_stale_links(Instance& in, int unused) {
+  auto stale = [&](dd_prec prec) { return !(in.links_fresh >> (int)prec & 1u) && in.links_unused[(int)prec] >= unused; };
+  bool any = false;
+  if (stale(DD_F64)) any |= drop_copy(in.link64_buf, in.d.link64);
+  if (stale(DD_F32)) any |= drop_copy(in.link32_buf, in.d.link32) | drop_copy(in.lb32_buf, in.d.lb32);
+  if (stale(DD_BF16)) any |= drop_copy(in.link16_buf, in.d.link16) | drop_copy(in.lb16_buf, in.d.lb16);
+  if (stale(DD_DF64)) any |= drop_copy(in.linkdf_buf, in.d.linkdf);
+  return any;
+}
+
+bool drop_clover_bundles(Instance& in) {
+  in.cb_gen = -1;
+  return drop_copy(in.cb32_buf, in.d.cb32);
+}
+
+// what an allocation short of memory gives back: link copies of an earlier gauge field, and clover
+// bundles of an earlier term (which clover_mixed_tables builds before their use, as ensure_links)
+static bool drop_stale_copies(dd_ctx* c) {
   bool any = false;
   for (auto& in : c->inst) {
-    auto drop = [&](dd_prec prec, void*& buf) {
-      if (!buf || (in.links_fresh >> (int)prec & 1u)) return;
-      dfree(buf);
-      buf = nullptr;
-      any = true;
-    };
-    drop(DD_F64, in.link64_buf);
-    drop(DD_F32, in.link32_buf);
-    drop(DD_F32, in.lb32_buf);
-    drop(DD_BF16, in.link16_buf);
-    drop(DD_BF16, in.lb16_buf);
-    drop(DD_DF64, in.linkdf_buf);
+    any |= drop_stale_links(in, 0);
+    if (in.cb_gen != c->clover_gen) any |= drop_clover_bundles(in);
   }
   return any;
+}
+
+// the links have changed: every copy is stale.  Those not used under the last `unused` fields are
+// given back.  A trajectory uses the frame's copies at its two ends only, so its updates of the
+// links keep unused ones for a while (freed at the second update and allocated again at the end
+// they made two steps on 16^4 take 70.2 ms, now 69.9).
+constexpr int UNUSED_UPLOADS = 1, UNUSED_UPDATES = 8;
+static void links_changed(dd_ctx* c, int unused) {
+  for (auto& in : c->inst) {
+    for (int p = 0; p < 4; ++p) in.links_unused[p] = in.links_fresh >> p & 1u ? 0 : in.links_unused[p] + 1;
+    drop_stale_links(in, unused);
+    in.links_fresh = 0;
+  }
+  c->links_settled = false;
+  c->inst_dirty = true;
 }
 
 dd_status dalloc(dd_ctx* c, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation && drop_stale_links(c)) {
+  const bool fault = c->alloc_fault > 0 && --c->alloc_fault == 0;      // test hook
+  cudaError_t e = fault ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && drop_stale_copies(c)) {
     cudaGetLastError();
     e = cudaMalloc(p, bytes);
   }
@@ -467,19 +503,15 @@ dd_status gauge_finish(dd_ctx* c) {
     DD_CUDA(c, cudaGetLastError());
   }
   DD_CUDA(c, cudaDeviceSynchronize());
-  for (auto& in : c->inst) in.links_fresh = 0;
-  c->links_settled = false;
+  links_changed(c, UNUSED_UPLOADS);
   c->gauge_ready = true;
-  c->inst_dirty = true;
   return clover_build(c);        // no-op without the clover term
 }
 
 // after links in d_U changed on the device (a molecular-dynamics update): every
 // gathered per-domain copy is stale (the stored links keep their time sign)
 void gauge_touched(dd_ctx* c) {
-  for (auto& in : c->inst) in.links_fresh = 0;
-  c->links_settled = false;
-  c->inst_dirty = true;
+  links_changed(c, UNUSED_UPDATES);
 }
 
 dd_status check_device_error(dd_ctx* c, cudaStream_t s) {
@@ -962,6 +994,12 @@ dd_status dd_roots(int N, double c, double* u) {
     u[2 * (k - 1)] = cos(ph);
     u[2 * (k - 1) + 1] = s * sin(ph);
   }
+  return DD_OK;
+}
+
+dd_status dd_debug_alloc_fault(dd_ctx* c, int k) {
+  if (!c || k < 0) return DD_EINVAL;
+  c->alloc_fault = k;
   return DD_OK;
 }
 

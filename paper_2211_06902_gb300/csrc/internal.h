@@ -70,6 +70,7 @@ struct Instance {
   std::vector<int> h_glob;      // host copy [p][n_p]
   std::vector<int> h_fmap;      // host copy [p][n_p]
   unsigned links_fresh = 0;     // bit per precision: that copy holds the current links
+  int links_unused[4] = {0, 0, 0, 0};   // gauge fields since that copy's last use
 };
 
 struct BlockDesc {
@@ -213,6 +214,7 @@ struct dd_ctx {
   bool links_settled = false;              // no kernel in flight reads copies of an earlier gauge field
   int forced_variant[3] = {-1, -1, -1};    // manual stencil launch variant per precision
   bool debug_wait_fault = false;           // test hook: see dd_debug_wait_fault
+  int alloc_fault = 0;                     // test hook: see dd_debug_alloc_fault
 };
 
 // ---- helpers shared by the translation units --------------------------------
@@ -290,6 +292,8 @@ dd_status gauge_finish(dd_ctx* c);
 // v <- A v or A^{-1} v on both parity vectors of a batch (FP64)
 dd_status clover_build(dd_ctx* c);
 void gauge_touched(dd_ctx* c);
+// frees the clover bundles of an instance; true if there were any
+bool drop_clover_bundles(Instance& in);
 dd_status clover_apply(dd_ctx* c, const Batch& b, void* ve, void* vo, bool inverse, cudaStream_t s);
 // the packed copies of A^{-1} that the mixed solves read: the double-float table and the
 // FP32 bundles of the batch's instances

@@ -126,6 +126,7 @@ def lib():
             "dd_set_clover": [vp, C.c_double],
             "dd_debug_wait_fault": [vp, C.c_int],
             "dd_debug_inner_sums": [vp, C.c_int, dp],
+            "dd_debug_alloc_fault": [vp, C.c_int],
             "dd_logdet_force": [vp, C.c_int, vp, vp, C.POINTER(SolveParams), vp],
             "dd_fp64_fma_rate": [dp],
             "dd_apply_w_part": [vp, C.c_int, C.c_int, ip, C.c_int, vp, vp, C.POINTER(SolveParams), vp],
@@ -154,7 +155,7 @@ def exported_symbols():
             "dd_net_apply", "dd_net_loss_grad", "dd_net_train", "dd_set_net", "dd_net_save", "dd_net_load", "dd_multiboson_heatbath",
             "dd_set_hop_variant", "dd_hop_variants", "dd_hop_variant_name",
             "dd_apply_D_block_noalloc", "dd_reweight_samples", "dd_mb_force", "dd_set_clover",
-            "dd_debug_wait_fault", "dd_debug_inner_sums", "dd_logdet_force", "dd_fp64_fma_rate", "dd_apply_w_part",
+            "dd_debug_wait_fault", "dd_debug_inner_sums", "dd_debug_alloc_fault", "dd_logdet_force", "dd_fp64_fma_rate", "dd_apply_w_part",
             "dd_net_tensor_cores", "dd_pf_heatbath", "dd_md_trajectory", "dd_clover_cond"]
 
 
@@ -488,6 +489,10 @@ class Context:
     def debug_wait_fault(self, on):
         """Test hook: the bundle-form stencil's bounded wait gives up (DD_ETIMEOUT)."""
         self._check(lib().dd_debug_wait_fault(self._h, 1 if on else 0))
+
+    def debug_alloc_fault(self, k):
+        """Test hook: the k-th device allocation from now on acts as if the device were out of memory."""
+        self._check(lib().dd_debug_alloc_fault(self._h, int(k)))
 
     def debug_inner_sums(self, nsys):
         """Test hook: inner target |r|^2 and last alpha of the last solve's systems, [nsys] and [nsys] complex."""
