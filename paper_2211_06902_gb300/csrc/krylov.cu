@@ -783,9 +783,13 @@ dd_status run_bicgstab(dd_ctx* c, const Batch& b, dd_prec prec, const InnerVecs&
 
 // Measures every compiled variant of the hop launch on this batch (the
 // H_oe half-apply of an initialised even vector `in` into `out`) and keeps
-// the fastest for the precision.
-dd_status tune_hop(dd_ctx* c, const Batch& b, dd_prec prec, const void* in, void* out,
-                   cudaStream_t s) {
+// the fastest for the precision.  In FP64 also H_eo with the inner products of
+// t = M s, into `out_e`: variant 0 takes another kernel for small bare hops than
+// for those with products (launch_hop), and half of a solve's hops are of either
+// kind (12^4, 2 rhs: variant 0 by the bare hop alone, 9917 us a solve; variant 1
+// by both, 9680).
+dd_status tune_hop(dd_ctx* c, const Batch& b, dd_prec prec, const void* in, void* out, void* out_e,
+                   double* partial, cudaStream_t s) {
   const int pi = prec == DD_F64 ? 0 : (prec == DD_F32 ? 1 : 2);
   const bool timing = c->timing;
   c->timing = false;
@@ -801,11 +805,18 @@ dd_status tune_hop(dd_ctx* c, const Batch& b, dd_prec prec, const void* in, void
     b.hop_variant[pi] = v;
     HopArgs h{};
     h.p_out = 1; h.in = in; h.out = out; h.b = 1.0;
-    for (int k = 0; k < 2 && st == DD_OK; ++k) st = launch_hop(c, b, prec, h, s);
+    HopArgs g{};
+    g.p_out = 0; g.in = out; g.out = out_e; g.s1 = in; g.a1 = 1.0; g.b = -c->kappa * c->kappa;
+    g.dots = in; g.dotq = in; g.dotqs = true; g.rhat_seed = BicgOps<double2>::rseed; g.partial = partial;
+    auto hops = [&]() {
+      if (st == DD_OK) st = launch_hop(c, b, prec, h, s);
+      if (st == DD_OK && prec == DD_F64) st = launch_hop(c, b, prec, g, s);
+    };
+    for (int k = 0; k < 2; ++k) hops();
     float vbest = 1e30f;
     for (int round = 0; round < 3 && st == DD_OK; ++round) {
       cudaEventRecord(e0, s);
-      for (int k = 0; k < 3 && st == DD_OK; ++k) st = launch_hop(c, b, prec, h, s);
+      for (int k = 0; k < 3; ++k) hops();
       cudaEventRecord(e1, s);
       cudaEventSynchronize(e1);
       float ms = 0;
@@ -1384,7 +1395,7 @@ dd_status solve_batch(dd_ctx* c, const Batch& b, const double* b_user, double* x
     if ((e = to_inner(s)) != DD_OK) return e;
     if ((prm->flags & DD_SOLVE_AUTOTUNE) && cyc == 0) {
       const int pi = ip == DD_F64 ? 0 : (ip == DD_F32 ? 1 : 2);
-      if (!b.tuned[pi] && (e = tune_hop(c, b, ip, rin_e, ip == DD_F64 ? tune64 : w.tmp, s)) != DD_OK)
+      if (!b.tuned[pi] && (e = tune_hop(c, b, ip, rin_e, ip == DD_F64 ? tune64 : w.tmp, w.v, partial, s)) != DD_OK)
         return e;
     }
     if ((e = schur_rhs(s)) != DD_OK) return e;
