@@ -600,8 +600,9 @@ dd_status dd_apply_D_block_noalloc(dd_ctx* ctx, dd_domain kind, const int* ids, 
 
 /* Measured FP64 fused multiply-add rate of the current device in TFLOP/s
  * (best of three timed launches of independent FMA chains on every SM, after
- * one warm-up launch; clocks as they are).  The ALU roofline of the FP64
- * kernels (the force contraction, the plain FP64 stencil).  No counterpart in
+ * one warm-up launch; clocks as they are): the rate of the FP64 pipes, two
+ * flops an instruction.  The ALU roofline of the FP64 kernels (the force
+ * contraction, the plain FP64 stencil).  No counterpart in
  * the paper.  Synchronises the legacy default stream. */
 dd_status dd_fp64_fma_rate(double* tflops);
 

@@ -500,8 +500,9 @@ __device__ __forceinline__ void force_link(const double2 (&U)[9], const double2*
 // fields, N = sum_f [ conj(U h(z(x+mu))) (x) h(y(x)) - conj(h(z(x))) (x) U h(y(x+mu)) ]
 // (half spinors of the backward / forward projectors, see force_link), T_t = lambda_t/2,
 // z = gamma_5 times the solution of the gamma_5-rotated adjoint system.
-// Bound by the FP64 pipe: 576 flops per link and field run at the measured FP64 FMA rate
-// (32^4, 12 fields: 13.6 ms, 1069 of 1058 GFLOP/s).
+// Bound by the FP64 pipe: 288 FMAs and 48 additions per link and field issue at 96 % of its rate
+// (24^4, 12 fields: 4.47 ms, 601 of 629 G instructions a second over all lanes; 92 % by ncu on 16^4
+// with 4 fields).
 // The plan lists a block's links direction by direction, so a warp takes one branch of the
 // switch; with the four directions of a site on neighbouring lanes each warp ran all four, and
 // the 24^4 lattice with 12 fields took 20.4 ms. Together with the outer products as two FMAs
