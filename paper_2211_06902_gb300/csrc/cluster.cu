@@ -14,6 +14,7 @@
 // layout and slots of the launched form.  8^4 x 4 rhs whole solve 2222 -> 1069 us, action
 // on 8^4 with 2 fields 4910 -> 2284 us.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "internal.h"
@@ -32,7 +33,7 @@ constexpr int CL_UBUF = 8 * 6 * 32;    // half-spinor numbers of one 32-site chu
 // An inner product adds four numbers a lane and step in FP32.  After six steps the lane has added
 // the 24 numbers that a site has in the launched form; the warp's sum of them (768 numbers, as
 // there) is set aside, and everything above is FP64.  A lane has one step on 8^4, seven with framed
-// 9^4 blocks and up to 36 on the largest batches taken; one FP32 sum over all of them was up to 72
+// 9^4 blocks and up to 34 on the largest frames taken; one FP32 sum over all of them was up to 72
 // units of FP32 rounding off where these are at most 30.  A run's end costs a lane about 100
 // instructions (16^4 x 4 rhs 4517 us a solve, without it 4417; 8^4 x 4 rhs has none).
 constexpr int CL_FP32_STEPS = 6;
@@ -604,16 +605,21 @@ void cluster_prepare() {
 //
 // A hop of a cluster takes steps of 32 sites x 1 rhs, one after the other in each group:
 // ceil(chunks / groups) * rb of them, about 1 us each alone on an SM and 1.25 us with two CTAs
-// per SM, in waves of 2 CTAs per SM.  rb and cs are those with the least time by this count
-// (measured against every rb <= 4 and cs in 2, 4, 8 on 8^4 .. 20^4 with 1 .. 12 rhs: within 7 %
-// of the best).  An iteration has four hops and about 12 us of barriers and reductions.
-// The launched form needs about 5 us + work / 9800 us a hop (work: even sites x rhs) and 14 us
-// of other launches, and streams from DRAM once the vectors outgrow L2: measured whole solves
-// (launched / one launch, us) 8^4 x 4 rhs 2233 / 982, 12^4 x 4 2890 / 1918, 16^4 x 1
-// 2704 / 2313, 16^4 x 4 5079 / 4442, 20^4 x 2 6615 / 5843, 24^4 x 1 7583 / 7033, but 8 uneven
-// blocks x 5 4626 / 5032, where the counts are 93 and 107 us an iteration; from about 400
-// thousand even sites x rhs on the two meet, so the line lies at 300 thousand.  Not taken with
-// the clover term, per-launch timing, a chosen launch form or the wait test, which concern the
+// per SM, in waves of 2 CTAs per SM.  On blocks of more than 8^4 sites neighbouring sites meet less
+// often in L1 and a step takes longer, 1.1 us on 9^4 and 3 on 13^4; frames and frame pieces miss
+// many of their hops and don't show that.  With one CTA per system a step takes 10 % longer (its
+// barriers have nothing to overlap), with BF16 vectors too.  rb and cs are those with the least time
+// by this count.  An iteration has four hops and about 12 us of barriers and reductions; the launched
+// form takes 36 us + work / 2500 (work: even sites x rhs), and streams from DRAM once the vectors
+// outgrow L2.  us an iteration, launched / one launch: blocks of 5^4 x 4 rhs 52 / 15, 7^4 x 4
+// 67 / 37, 9^4 x 1 63 / 55, 9^4 x 4 121 / 103, frame of 12^4 with 12 rhs 55 / 35, 81 blocks of
+// 7^4 x 2 113 / 94; launched are, among others, 10^4 x 1 70 / 76, 11^4 x 1 110 / 120, 13^4 x 1
+// 176 / 241 (BF16 140 / 265), which a rule without the blocks' size gave to the one launch.  Over 140
+// batches of 1 .. 81 systems with 1 .. 16 rhs the form taken is at most 1 % slower an iteration than
+// the other (2 % in whole solves of uneven blocks, whose systems end at different times).
+// From about 400 thousand even sites x rhs on the two meet, so the line lies at 300 thousand.
+// Not taken with the clover term (its A^-1 is bulk-copied beside the link bundles, which has no place
+// in this kernel), per-launch timing, a chosen launch form or the wait test, which concern the
 // launched kernels.
 ClusterPlan cluster_plan(dd_ctx* c, const Batch& b, dd_prec prec) {
   const ClusterPlan none{0, 0};
@@ -623,23 +629,27 @@ ClusterPlan cluster_plan(dd_ctx* c, const Batch& b, dd_prec prec) {
   const double work = (double)b.tot[0] / 12.0;
   if (work > 3e5) return none;
   const int nq = (std::max(b.maxn[0], b.maxn[1]) + 31) / 32;
+  // a step on whole blocks: their mean number of even sites against that of 9^4
+  double big = 1.08 * std::pow(work / ((double)b.nrhs * b.nb) / 3281.0, 0.7);
+  for (int j : b.inst)
+    if (c->inst[j].d.kind != DD_DOMAIN_OMEGA && c->inst[j].d.kind != DD_DOMAIN_FULL) big = 0.0;
   ClusterPlan best = none;
   double tbest = 0.0;
   for (int rb = std::min(b.nrhs, CL_R); rb >= 1; --rb) {
     const long long ng = (b.nrhs + rb - 1) / rb;
     for (int cs = 1; cs <= 8; cs *= 2) {
+      if (cl_runs(cl_steps(nq, cs)) > CL_MAX_RUNS) continue;   // 37 steps and more are never the faster form
       const long long ctas = b.nb * ng * cs;
       const double waves = (double)((ctas + 2LL * c->nsm - 1) / (2LL * c->nsm));
-      if (cl_runs(cl_steps(nq, cs)) > CL_MAX_RUNS) continue;   // 37 steps and more are never the faster form
-      const double steps = (double)cl_steps(nq, cs) * rb;
-      const double t = waves * (4.0 * steps * (ctas > c->nsm ? 1.25 : 1.0) + 12.0);
+      const double step = std::max(ctas > c->nsm ? 1.25 : 1.0, big) * (cs == 1 ? 1.1 : 1.0);
+      const double t = waves * (4.0 * cl_steps(nq, cs) * rb * step + 12.0) * (prec == DD_BF16 ? 1.1 : 1.0);
       if (best.cs == 0 || t < tbest) {
         best = {rb, cs};
         tbest = t;
       }
     }
   }
-  return tbest < 4.0 * (5.0 + work / 9800.0) + 14.0 ? best : none;
+  return tbest < 36.0 + work / 2500.0 ? best : none;
 }
 
 dd_status run_cluster(dd_ctx* c, const Batch& b, dd_prec prec, ClusterPlan plan, const void* rhs, void* x, void* r,

@@ -1,4 +1,4 @@
-"""Rounding of the inner solver's products on blocks of many 32-site chunks.
+"""Rounding of the inner solver's products on systems of many 32-site chunks.
 
 A lane adds at most 24 numbers in FP32, a warp 32 lanes in five more additions, and everything above is FP64, in the
 launched form and in the one-launch form of small batches.  At kappa = 0 the Schur complement is the identity: the
@@ -14,8 +14,8 @@ from paper_2211_06902_gb300 import dd4d, synth
 pytestmark = pytest.mark.gpu
 
 U = 2.0 ** -24                       # unit roundoff of FP32
-CELL, SIDE = 12, 13                  # 16 framed blocks of 13^4: 447 chunks of the even sites
-CHUNKS = 447
+RHS = 16                             # on the frame of 16^4 with 7^4 cores: 424 chunks of its even sites
+CHUNKS = 424
 
 
 def _mix32(x):
@@ -37,13 +37,14 @@ def _shadow(system, n, comps):
 
 @pytest.fixture(scope="module")
 def case():
-    ctx = dd4d.Context((2 * CELL,) * 4, 0.0)
+    L = (16,) * 4
+    ctx = dd4d.Context(L, 0.0)
     ctx.gauge_random(0.3, 1)
-    info = ctx.set_geometry([[(0, CELL - 2), (CELL, 2 * CELL - 2)]] * 4)
-    assert info["nblocks"] == 16 and info["max_omega"] == SIDE ** 4
-    even = np.flatnonzero(np.indices((SIDE,) * 4).sum(axis=0).ravel() % 2 == 0)
+    ctx.set_geometry([[(0, 6), (8, 14)]] * 4)
+    sites = ctx.geom_sites(dd4d.SET_LAMBDA1)
+    even = np.flatnonzero(sum(np.unravel_index(sites, L)) % 2 == 0)
     assert (len(even) + 31) // 32 == CHUNKS
-    yield ctx, even
+    yield ctx, len(sites), even
     ctx.close()
 
 
@@ -51,23 +52,23 @@ def _solve(ctx, form, b):
     ctx.set_hop_variant("f32", 0 if form == "launched" else -1)
     x = np.zeros_like(b)
     c0 = dd4d.launch_count()
-    st = ctx.solve_blocks("omega", list(range(16)), 1, b, x,
+    st = ctx.solve_blocks("lambda1", None, RHS, b, x,
                           dd4d.params(1e-5, inner_prec="f32", inner_tol=0.5, maxiter=1, max_outer=1))
     launches = dd4d.launch_count() - c0
     assert st["status"] == dd4d.DD_OK and st["max_iters"] == 1
-    return launches, ctx.debug_inner_sums(16)
+    return launches, ctx.debug_inner_sums(RHS)
 
 
 @pytest.mark.parametrize("groups", [2, 4, 8, 16])    # chunks go to 2 groups of warps per CTA of a cluster of 1 .. 8
 @pytest.mark.parametrize("form", ["one launch", "launched"])
 def test_norms_of_long_vectors(case, form, groups):
-    ctx, even = case
+    ctx, n, even = case
     run = -(-CHUNKS // groups)
     first = np.arange(len(even)) // 32 % run == 0
     # four numbers 1 in a lane's first chunk and pair, then numbers below half an ulp of their sum
     v = np.where(first, 1.0, float(np.float32(np.sqrt(0.9 * 2.0 ** -22))))
-    b = np.zeros((16, 1, SIDE ** 4, 12), dtype=np.complex128)
-    b[:, 0, even] = (v * (1 + 1j))[None, :, None]
+    b = np.zeros((1, RHS, n, 12), dtype=np.complex128)
+    b[0, :, even] = (v * (1 + 1j))[:, None, None]
     _, (target, _) = _solve(ctx, form, b)
     exact = 0.25 * 24.0 * np.sum(v ** 2)
     # 24 additions in a lane and 5 in a warp, each off by at most U of the sum of positive numbers so far
@@ -77,14 +78,14 @@ def test_norms_of_long_vectors(case, form, groups):
 @pytest.mark.parametrize("groups", [2, 4, 8, 16])
 @pytest.mark.parametrize("form", ["one launch", "launched"])
 def test_products_of_long_vectors(case, form, groups):
-    ctx, even = case
+    ctx, n, even = case
     run = -(-CHUNKS // groups)
     first = np.arange(len(even)) // 32 % run == 0
     t = np.where(first, 1.0625, 0.9 * 2.0 ** -23)    # real part of conj(r^) b per component; the imaginary part is 0
-    b = np.zeros((16, 1, SIDE ** 4, 12), dtype=np.complex128)
-    for s in range(16):
+    b = np.zeros((1, RHS, n, 12), dtype=np.complex128)
+    for s in range(RHS):
         h = _shadow(s, len(even), 2)
-        b[s, 0, even, :2] = (t[:, None] * h / np.abs(h) ** 2).astype(np.complex64)
+        b[0, s, even, :2] = (t[:, None] * h / np.abs(h) ** 2).astype(np.complex64)
     _, (_, alpha) = _solve(ctx, form, b)
     # (r^, r) and (r^, M p) hold the same products in different order.  Of a lane's 24 numbers the two large components
     # are four, 2.125 together, and the other twenty ten small components: they lose at most 10 * 1.8 U / 2.125 = 8.5 U.
@@ -95,7 +96,7 @@ def test_products_of_long_vectors(case, form, groups):
 
 def test_both_forms_run(case):
     """Start (2 launches), one iteration (9) and the last check against one launch."""
-    ctx, even = case
-    b = np.zeros((16, 1, SIDE ** 4, 12), dtype=np.complex128)
-    b[:, 0, even] = 1
+    ctx, n, even = case
+    b = np.zeros((1, RHS, n, 12), dtype=np.complex128)
+    b[0, :, even] = 1
     assert _solve(ctx, "launched", b)[0] - _solve(ctx, "one launch", b)[0] == 11

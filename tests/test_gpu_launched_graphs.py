@@ -58,3 +58,25 @@ def test_without_a_chosen_variant_the_batch_takes_one_launch(inner):
     # both within cond(D) * tol of the solution; cond(D) < 100 at this kappa
     assert np.linalg.norm(x1 - x0) <= 2 * 100 * 1e-10 * np.linalg.norm(x0)
     ctx.close()
+
+
+@pytest.mark.parametrize("cell,nrhs,kind,inner,one", [
+    (4, 12, "omega", "f32", True), (8, 4, "omega", "f32", True), (6, 12, "lambda1", "f32", True), (10, 2, "omega", "f32", True),
+    (10, 1, "omega", "f32", False), (10, 1, "omega", "bf16", False), (12, 1, "omega", "f32", False),
+    (12, 1, "omega", "bf16", False), (9, 1, "omega", "bf16", False),
+])
+def test_form_of_small_batches(cell, nrhs, kind, inner, one):
+    """Where the one launch was measured faster, with a margin, it is taken; where the launched form was, that is."""
+    ctx = dd4d.Context((2 * cell,) * 4, 0.125)
+    ctx.gauge_random(0.5, 2)
+    info = ctx.set_geometry([[(0, cell - 2), (cell, 2 * cell - 2)]] * 4)
+    ids = list(range(info["nblocks"])) if kind == "omega" else None
+    n = info["nblocks"] * info["max_omega"] if ids else info["n_lambda1"]
+    b = synth.complex_gaussian(3, synth.TAG_RHS, (n * nrhs, 12))
+    x = np.zeros_like(b)
+    for call in range(2):                            # the first also gathers the links
+        n0 = dd4d.launch_count()
+        st = ctx.solve_blocks(kind, ids, nrhs, b, x, dd4d.params(1e-8, inner_prec=inner, inner_tol=1e-3))
+        n1 = dd4d.launch_count()
+    assert st["status"] == 0 and (n1 - n0 < 9 * st["max_iters"]) == one, (n1 - n0, st["max_iters"])
+    ctx.close()
