@@ -1221,9 +1221,12 @@ int hop_variant_count(dd_prec prec) { return prec == DD_F64 ? 5 : (prec == DD_F3
 // x rhs on, where the CTAs' start-up no longer shows (FP32 solves, plain / bundle form, ms: 24^4 x
 // 12 rhs 51.2 / 48.4 and x 8 35.8 / 34.8 and x 6 28.1 / 27.7, but x 4 20.3 / 21.4; 20^4 x 12
 // 27.3 / 26.7; 16^4 x 12 12.8 / 13.1).  Whole items of 12 rhs fill a CTA, fewer run better by halves.
+// The registers of an SM hold 25 warps: CTAs of 6, 8 or 12 warps (a warp per rhs) use 24 of them, of
+// 7 only 21 and of 9 only 18, and the plain form is faster (24^4, bundle form over plain: 7 rhs 1.03,
+// 9 rhs 1.06, 13 = 7 + 6 1.02, 17 = 9 + 8 1.07; but 6 rhs 1.00, 8 0.985, 10 0.99, 11 0.97, 12 0.95).
 int hop_default_f32(long long even_site_rhs, int nrhs) {
   const int ngroups = (nrhs + LB_MAX_RHS - 1) / LB_MAX_RHS, rb = (nrhs + ngroups - 1) / ngroups;
-  if (even_site_rhs < 1200000 || rb < 6) return 0;
+  if (even_site_rhs < 1200000 || rb < 6 || rb == 7 || rb == 9) return 0;
   return rb >= 10 ? 13 : 17;
 }
 

@@ -44,3 +44,22 @@ def test_stencil_before_and_after_a_tuned_solve(prec, nrhs):
         u = {"f64": 2.0 ** -53, "f32": 2.0 ** -24}[prec]
         assert np.abs(tuned - fresh).max() <= 64 * u * np.abs(fresh).max()
     ctx.close()
+
+
+@pytest.mark.parametrize("nrhs,starts", [(5, "k_hop<"), (6, "k_hop_lb"), (7, "k_hop<"), (8, "k_hop_lb"), (9, "k_hop<"),
+                                         (12, "k_hop_lb"), (13, "k_hop<"), (17, "k_hop<"), (18, "k_hop<")])
+def test_default_form_of_large_batches(nrhs, starts):
+    """Bundle CTAs have a warp per rhs; with 7 or 9 they leave much of an SM idle and the plain form is taken."""
+    torch = pytest.importorskip("torch")
+    ctx = dd4d.Context((24,) * 4, 0.12)
+    ctx.gauge_random(0.4, 2)
+    info = ctx.set_geometry([[(0, 6), (8, 14), (16, 22)]] * 4)
+    ids = list(range(info["nblocks"]))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(nrhs)
+    b = torch.randn((len(ids), nrhs, info["max_omega"], 24), generator=gen, device="cuda", dtype=torch.float64)
+    x = torch.zeros_like(b)
+    st = ctx.solve_blocks("omega", ids, nrhs, b, x, dd4d.params(1e-6, inner_prec="f32", inner_tol=1e-3))
+    assert st["status"] == 0 and st["max_relres"] <= 1e-6
+    assert dd4d.hop_variant_name("f32", st["hop_variant"]).startswith(starts)
+    ctx.close()
