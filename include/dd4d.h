@@ -96,12 +96,19 @@ typedef struct {
                           solve at that precision with FP64 defect correction */
   double inner_tol;    /* relative reduction per inner solve (mixed only), e.g. 1e-5 */
   int max_outer;       /* defect-correction cycles cap (mixed only) */
-  int check_every;     /* iterations between host convergence checks (>= 1) */
+  int check_every;     /* iterations between host convergence checks (>= 1); see below
+                          for small batches */
   int flags;           /* DD_SOLVE_* below, or-ed, or 0 */
   int restart;         /* Arnoldi steps per FGMRES cycle (DD_SOLVE_FGMRES; 1..16) */
 } dd_solve_params;
 
-/* dd_solve_params.flags */
+/* dd_solve_params.flags.  The inner BiCGstab of a small mixed batch (up to 300
+ * thousand even sites x rhs, without the clover term; the choice is the
+ * library's) runs as one launch that checks its own convergence: DD_SOLVE_GRAPH,
+ * DD_SOLVE_GRAPH_LOOP and check_every then have nothing to act on, and the
+ * tuned variant serves the hops outside of the inner solves only.  A launch
+ * variant chosen with dd_set_hop_variant, or kernel timing, makes such a batch
+ * run the launched iterations of the larger ones. */
 #define DD_SOLVE_GRAPH 1     /* replay the inner iterations between two host polls as one
                                 captured CUDA graph (ignored while kernel timing is on) */
 #define DD_SOLVE_AUTOTUNE 2  /* on a batch's first solve, time every compiled launch variant
@@ -141,7 +148,8 @@ typedef struct {
   int outer_cycles;    /* defect-correction cycles run (1 for plain FP64) */
   double max_relres;   /* largest final |b - D x|/|b|, FP64, over systems */
   double seconds;      /* device time of the call (CUDA events) */
-  int hop_variant;     /* stencil launch variant used at the inner precision (autotuner) */
+  int hop_variant;     /* stencil launch variant used at the inner precision (default, tuned or
+                          chosen); where the inner solves are one launch, of the hops around them */
 } dd_solve_stats;
 
 /* ---- context --------------------------------------------------------- */
@@ -172,10 +180,10 @@ dd_status dd_set_kappa(dd_ctx* ctx, double kappa);
  * tables), so the true residual stays within tol.  Every hop of a solve applies
  * A^{-1} of its output site at its own precision: FP64 for DD_F64 solves; for
  * DD_F32 and DD_BF16 inner solves an FP32 copy of A^{-1} (each hermitian block
- * packed to its diagonal and upper triangle, 288 B per site), and for their
- * double-float residual a double-float copy (576 B per site); A^{-1} b is
- * formed once in FP64.  The two copies (1.5 times the FP64 table) are built
- * at the first mixed solve after A changes.  dd_mb_force, dd_apply_D_block at
+ * packed to its diagonal and upper triangle, 288 B per site of every domain
+ * solved on), and for their double-float residual a double-float copy (576 B per
+ * lattice site); A^{-1} b is formed once in FP64.  Both are built at the first
+ * mixed solve after A changes.  dd_mb_force, dd_apply_D_block at
  * DD_F32 / DD_BF16, dd_apply_D_block_noalloc and the learned network
  * (DD_SOLVE_NET_GUESS, DD_SOLVE_NET_PRECOND) return DD_EINVAL with the term
  * on.  c_sw = 0 turns it off (the default)
@@ -267,8 +275,8 @@ dd_status dd_solve_blocks(dd_ctx* ctx, dd_domain kind, const int* ids, int nblk,
  * for every batch used afterwards on the context, overriding the autotuner;
  * v = -1 returns to the defaults.  Variants differ in launch shape (resident
  * CTAs per SM, persistent grid, rhs per thread, direction split, links staged
- * in shared memory by bulk copy), not in the per-site arithmetic; the fused
- * inner products may sum in a different order.  dd_hop_variant_name returns
+ * in shared memory by bulk copy), not in the per-site arithmetic; the eight
+ * directions and the fused inner products may sum in a different order.  dd_hop_variant_name returns
  * a static description of variant v (NULL if out of range). */
 dd_status dd_set_hop_variant(dd_ctx* ctx, dd_prec prec, int v);
 
@@ -562,7 +570,9 @@ dd_status dd_set_net(dd_ctx* ctx, dd_net* net);
 /* ---- kernel timing -----------------------------------------------------
  * With timing on, the library brackets every launch of its stencil kernels
  * with CUDA events on the launching stream, and so every launch of the force
- * kernel of dd_mb_force.  dd_timing_get returns, for kernel class `which`
+ * kernel of dd_mb_force.  Solves then run their launched, host-driven form: no
+ * graphs, and no one-launch inner solves of small batches, whose stencil is
+ * inside that launch and has no time of its own.  dd_timing_get returns, for kernel class `which`
  * (0: FP64 hop, 1: FP32 hop, 2: BF16 hop, 3: force), the summed device time
  * in ms, the number of launches and the summed algorithmic bytes (class 3:
  * algorithmic FP64 flops, 576 per active link and field: 72 complex

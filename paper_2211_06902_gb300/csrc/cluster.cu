@@ -9,10 +9,10 @@
 // step instead of eight, the links of a chunk serve the cluster's right-hand sides from
 // registers, and the warps' loads of neighbouring sites meet in L1.  The half spinors are
 // summed through shared memory.  What is left is latency on the smallest batches (8^4 x 4
-// rhs: 19 us an iteration) and the issue rate on larger ones (about 2000
+// rhs: 15 us an iteration) and the issue rate on larger ones (about 2000
 // warp instructions per step of a group).  Vectors stay in global memory (L2), in the
-// layout and slots of the launched form.  8^4 x 4 rhs whole solve 2222 -> 1069 us, action
-// on 8^4 with 2 fields 4910 -> 2284 us.
+// layout and slots of the launched form.  Against the launched form, all else as now: 8^4 x 4 rhs
+// whole solve 2206 -> 925 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

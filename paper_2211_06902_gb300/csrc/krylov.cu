@@ -6,8 +6,9 @@
 // and the even system is solved by BiCGstab (van der Vorst 1992) inside an
 // FP64 defect-correction loop: the outer residual r = b^_e - M x_e is always
 // formed in FP64; the inner BiCGstab runs at FP64 (plain form) or at
-// FP32 / BF16 storage with FP32 arithmetic (mixed forms) and FP64 inner
-// products.  All per-system scalars live on the device; the host only polls
+// FP32 / BF16 storage with FP32 arithmetic (mixed forms).  Its inner products
+// add a site's 24 numbers and the sites of a warp in FP32, the warps in FP64
+// (all in FP64 in the plain form).  All per-system scalars live on the device; the host only polls
 // the number of unconverged systems every `check_every` iterations.
 #include <algorithm>
 #include <functional>

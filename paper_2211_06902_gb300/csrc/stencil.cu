@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(HOP_THREADS, MINB) k_hop(BatchDev bd, HopArgs 
 }
 
 // The plain form on TH of an item's 128 sites per CTA, without inner products.  FP64 is bound by
-// the FP64 pipes (about 750 instructions a site, 17 cycles a warp), so the CTAs have to cover all
+// the FP64 pipes (about 750 instructions a site, 16 cycles a warp instruction), so the CTAs have to cover all
 // SMs evenly: 16 blocks of 5^4 with one rhs are 48 items, which kept 48 SMs busy for 27 us a hop
 // (FP64 stencil call there 83.1 us, now 73.9).  USER: the output leaves in the caller layout, which
 // saves dd_apply_D_block a pass over it (FP32, 24^4 x 12 rhs: 1201 us a call, now 1060).
